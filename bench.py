@@ -141,13 +141,16 @@ INTERIOR_SOURCES = ("tlbm_device.cuh", "tlbm_kernels.cuh", "tlbm_ops.h", "tlbm_o
 
 
 def kernel_source_hash():
-    """SHA-256 over the sources of the interior kernel, to tell whether a
-    stored ncu capture still describes the kernel being timed."""
+    """SHA-256 over the sources of the interior kernel without their comments
+    and blank lines, to tell whether a stored ncu capture still describes the
+    kernel being timed."""
     import hashlib
+    import re
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_1710_09534_gb300", "csrc")
     for f in INTERIOR_SOURCES:
-        h.update(open(os.path.join(csrc, f), "rb").read())
+        text = re.sub(r"/\*.*?\*/|//[^\n]*", "", open(os.path.join(csrc, f)).read(), flags=re.S)
+        h.update("\n".join(line.rstrip() for line in text.splitlines() if line.strip()).encode())
     from paper_1710_09534_gb300 import build
     fl = build._flags()
     # the compiler flags shape the code too (the include paths, which depend on

@@ -383,14 +383,15 @@ int tlb_set_params(tlb_lattice* L, const tlb_params* p)
         P.k34Dlam[i] = 0.75 * p->D * P.lam[i];
         P.eta[i] = M[i] / ((1.0 / 3.0) * (tau[i] - 0.5));
         P.inv_tau[i] = 1.0 / tau[i];
-        P.omt[i] = 1.0 - 1.0 / tau[i];
-        P.src_f[i] = 3.0 * (1.0 - 0.5 / tau[i]);
-        P.e0[i] = (4.0 / 9.0 - 1.0) * P.eta[i] / tau[i];
-        for (int c = 0; c < 2; c++) {
-            P.aw[i][c] = P.eta[i] * w[c] / tau[i];
-            P.bw[i][c] = 3.0 * w[c] / tau[i];
-            P.sw[i][c] = P.src_f[i] * w[c];
-        }
+        // relaxation time of the order parameters' common rate
+        const double t = mrt ? 1.0 / p->mrt_s_f : tau[i];
+        P.rate[i] = 1.0 / t;
+        P.kj[i] = mrt ? (p->mrt_s_f - P.inv_tau[i]) / 6.0 : 0.0;
+        P.omt[i] = 1.0 - 1.0 / t;
+        P.e0[i] = (4.0 / 9.0 - 1.0) * P.eta[i] / t;
+        P.kq[i] = 3.0 / 36.0 / t;
+        P.ks[i] = 3.0 * (1.0 - 0.5 / t) / 36.0;
+        for (int c = 0; c < 2; c++) P.aw[i][c] = P.eta[i] * w[c] / t;
     }
     P.rho[0] = p->rho1;
     P.rho[1] = p->rho2;
@@ -434,9 +435,6 @@ int tlb_set_params(tlb_lattice* L, const tlb_params* p)
         P.K34l6[i] = P.k34Dlam[i] / 6.0;
         P.drho12[i] = P.drho[i] / 12.0;
         P.aM6[i] = P.aM[i] / 6.0;
-        P.k3tau[i] = 3.0 / tau[i];
-        P.kq[i] = 3.0 / 36.0 / tau[i];
-        P.ks[i] = P.src_f[i] / 36.0;
         P.K3w3[i] = 3.0 * P.Kw3[i];
     }
     P.Kt = P.k12D * P.two_lamT;

@@ -45,7 +45,7 @@ k_batch_interior(const LatDesc<R>* __restrict__ descs, const TileItem* __restric
                  BatchCounters* __restrict__ ctr, int parity)
 {
     __shared__ ColRings<R, BLOCK> sh;
-    constexpr bool kStash = kStashPops && std::is_same<R, float>::value && !MRT;
+    constexpr bool kStash = kStashPops && std::is_same<R, float>::value && !kDenseMrt<S, MRT>;
     __shared__ PopStash<R, kStash ? BLOCK : 1> stash;
     __shared__ Prm<R> Ps;
     __shared__ int item_s;

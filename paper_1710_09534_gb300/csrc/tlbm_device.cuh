@@ -51,12 +51,11 @@ struct Prm {
     R k4D;            // 4 / D (Eq. 42 with dx = 1)
     R eta[2];         // eta_i = M_i / (cs^2 (tau_i - 1/2))
     R inv_tau[2];     // 1 / tau_i
+    // omt, e0, aw, kq, ks: with the MRT collision, the same with rate_i in the
+    // place of 1 / tau_i (Collider adds the flux moments' difference)
     R omt[2];         // 1 - 1 / tau_i
-    R src_f[2];       // (1 - 1/(2 tau_i)) * 3 (Eq. 11a with 1/cs^2)
     R e0[2];          // (w_0 - 1) eta_i / tau_i  (k = 0 equilibrium, relaxed)
     R aw[2][2];       // eta_i w_c / tau_i
-    R bw[2][2];       // 3 w_c / tau_i
-    R sw[2][2];       // src_f_i w_c
     R rho[3], nu[3];
     R drho[2], dnu[2];  // rho_i - rho_3, nu_i - nu_3
     R aM[2];          // (rho_i - rho_3) M_i (Eq. 12)
@@ -67,6 +66,8 @@ struct Prm {
     R mrt;            // 1: MRT collision (moment basis below), 0: BGK
     R mrt_s_f;        // MRT rate of the non-flux moments of f^i
     R mrt_s_g;        // MRT rate of the energy moments of g
+    R rate[2];        // rate of the order-parameter relaxation: 1 / tau_i, MRT: mrt_s_f
+    R kj[2];          // (mrt_s_f - 1 / tau_i) / 6 (MRT: the flux moments' own rate)
     // equal densities and equal viscosities (rho_i = rho_3, nu_i = nu_3): the
     // constants the uniform-property update uses instead of per-node values
     R uni;            // 1 when both hold
@@ -81,8 +82,7 @@ struct Prm {
     R qa[2][2];       // F_s weights: (mu_i - mu_3) / 12 = qa[i][0] mu_1 + qa[i][1] mu_2
     R drho12[2];      // (rho_i - rho_3) / 12
     R aM6[2];         // (rho_i - rho_3) M_i / 6
-    R k3tau[2];       // 3 / tau_i
-    R kq[2], ks[2];   // 3 w36 / tau_i, w36 src_f_i (the order-parameter sources per w36)
+    R kq[2], ks[2];   // 3 w36 / tau_i, 3 w36 (1 - 1/(2 tau_i)) (order-parameter sources, Eqs. 2a, 11a)
     R K3w3[2];        // 3 Kw3 (uniform properties: K_w T = K3w3 (F_s + G))
 };
 
@@ -262,8 +262,25 @@ __device__ __forceinline__ void hydro_from_g(const Prm<R>& P, const Macro<R>& m,
 // V_i is formed per pair from Q'_i = w36 Q_i: 4 Q'_x or 4 Q'_y on the axis
 // links (w_axis = 4 w36, folded into one fma with A_i), Q'_x +- Q'_y on the
 // diagonal ones.
-template <typename R, bool UNI = false>
+//
+// MRT (FP64): the moment-space relaxation differs from the
+// BGK one in few moments, so it is the BGK update with one rate per
+// distribution plus the rank-2 and rank-4 differences, M^-1 being the
+// transposed basis over its squared norms (basis rows as in mrt_m below):
+//   f^i: rate s_f in every moment; the flux moments j_x, j_y relax at 1/tau_i
+//     instead, which adds e_k . D_i, D_i = (s_f - 1/tau_i)/6 (j - c_i u + d_i/2)
+//     with d_i = d/dt(c_i u) (sum_k e_k f^eq_k = c_i u, sum_k e_k src_k = d_i);
+//     the conserved moment has no non-equilibrium part;
+//   g: rate 1/tau_g in every moment; r in (e, eps, q_x, q_y) relaxes at s_g
+//     instead, which adds M^-1_kr dl_r, dl_r = -(s_g - 1/tau_g)(m_r(g) - X_r),
+//     X_r = m_r(g^eq) - m_r(src)/2 in closed form (build).
+// What bounds the FP64 update is its FP64 instructions: two dense 9x9 moment
+// transforms per distribution (and per source) took about 1100 per node
+// against 220 for BGK; this form adds about 85.  GB300, 777x501, FP64:
+// 858 -> 316 us per step.
+template <typename R, bool UNI = false, bool MRT = false>
 struct Collider {
+    static constexpr bool kMrt = MRT;
     R A1[2], A2[2];     // per class (0 axis, 1 diagonal)
     R Q1[2], Q2[2];     // w36 Q_i (x, y)
     R E1, E2;           // f^{i,eq}_0 / tau_i
@@ -272,6 +289,11 @@ struct Collider {
     R KX[4], RX[2], PX[2], AX[4];
     R omt1, omt2, omtg;
     R P0;               // g^eq_0 / tau_g + G_0
+    // MRT only: X_r and the rate difference of g; (kj, c_i u - d_i/2) of f^i,
+    // then D_i and Q'_i + D_i
+    R Xr[4], dsg;
+    R kj[2], jq[2][2];
+    R D1[2], D2[2], Qd1[2], Qd2[2];
 
     // SE: the moving populations and g_0 are handled in units of 2^SE (see
     // collide_all); the constants that add to them are scaled to match.
@@ -283,8 +305,8 @@ struct Collider {
         // order parameters
         omt1 = P.omt[0];
         omt2 = P.omt[1];
-        E1 = fma(P.e0[0], m.mu1, P.inv_tau[0] * m.c1);
-        E2 = fma(P.e0[1], m.mu2, P.inv_tau[1] * m.c2);
+        E1 = fma(P.e0[0], m.mu1, P.rate[0] * m.c1);
+        E2 = fma(P.e0[1], m.mu2, P.rate[1] * m.c2);
 #pragma unroll
         for (int c = 0; c < 2; c++) {
             A1[c] = P.aw[0][c] * m.mu1;
@@ -357,6 +379,22 @@ struct Collider {
         // k = 0: g^eq_0 = 3p (w0 - 1) + rho w0 t0; G_0 = -w0 kG (t0 u.H + u.T)
         const R geq0 = fma(m.rho * w0, t0, R(3) * (w0 - R(1)) * h.p);
         P0 = fma(geq0, itg, -(w0 * kG) * fma(t0, uH, uT));
+        if constexpr (MRT) {
+            static_assert(SE == 0, "the MRT update works in plain units");
+            dsg = P.mrt_s_g - itg;
+            const R Hx = h.grx + R(3) * h.Ftx, Hy = h.gry + R(3) * h.Fty;
+            const R ru = R(3) * m.rho * h.usq, uu = R(1.5) * h.usq * uH, uxy = h.ux * h.uy;
+            Xr[0] = fma(R(6), h.p, ru) + (uu - uT);
+            Xr[1] = fma(R(0.5), uH + uT, -fma(R(9), h.p, ru)) - uu;
+            Xr[2] = fma(R(0.5), fma(-h.uy * h.uy, Hx, h.Ftx), -fma(m.rho, h.ux, uxy * Hy));
+            Xr[3] = fma(R(0.5), fma(-h.ux * h.ux, Hy, h.Fty), -fma(m.rho, h.uy, uxy * Hx));
+            kj[0] = P.kj[0];
+            kj[1] = P.kj[1];
+            jq[0][0] = fma(m.c1, h.ux, R(-0.5) * d1x);
+            jq[0][1] = fma(m.c1, h.uy, R(-0.5) * d1y);
+            jq[1][0] = fma(m.c2, h.ux, R(-0.5) * d2x);
+            jq[1][1] = fma(m.c2, h.uy, R(-0.5) * d2y);
+        }
         if constexpr (SE != 0) {
             constexpr R sc = R(1 << SE);
 #pragma unroll
@@ -377,6 +415,39 @@ struct Collider {
         }
     }
 
+    // MRT: the energy moments' difference of g, folded into the constants that
+    // add to its populations
+    __device__ __forceinline__ void moments_of_g(const R g[9])
+    {
+        const R ax = (g[1] + g[3]) + (g[2] + g[4]), dg = (g[5] + g[7]) + (g[6] + g[8]);
+        const R d57 = g[5] - g[7], d86 = g[8] - g[6];
+        const R k36 = dsg * R(-1.0 / 36.0), k12 = dsg * R(-1.0 / 12.0);
+        const R de = k36 * (fma(R(-4), g[0], fma(R(2), dg, -ax)) - Xr[0]);
+        const R dp = k36 * (fma(R(4), g[0], fma(R(-2), ax, dg)) - Xr[1]);
+        const R dx = k12 * (fma(R(-2), g[1] - g[3], d57 + d86) - Xr[2]);
+        const R dy = k12 * (fma(R(-2), g[2] - g[4], d57 - d86) - Xr[3]);
+        P0 = fma(R(4), dp - de, P0);
+        PX[0] -= fma(R(2), dp, de);
+        PX[1] += fma(R(2), de, dp);
+        AX[0] = fma(R(-2), dx, AX[0]);
+        AX[1] = fma(R(-2), dy, AX[1]);
+        AX[2] += dx + dy;
+        AX[3] += dx - dy;
+    }
+    // MRT: D_i from the first moments (jx, jy) of f^1 and f^2
+    __device__ __forceinline__ void flux_of_f(R j1x, R j1y, R j2x, R j2y)
+    {
+        D1[0] = kj[0] * (j1x - jq[0][0]);
+        D1[1] = kj[0] * (j1y - jq[0][1]);
+        D2[0] = kj[1] * (j2x - jq[1][0]);
+        D2[1] = kj[1] * (j2y - jq[1][1]);
+#pragma unroll
+        for (int c = 0; c < 2; c++) {
+            Qd1[c] = Q1[c] + D1[c];
+            Qd2[c] = Q2[c] + D2[c];
+        }
+    }
+
     // rest direction
     __device__ __forceinline__ void post0(R f10, R f20, R g0, R& o1, R& o2, R& og) const
     {
@@ -393,7 +464,20 @@ struct Collider {
         static_assert(K == 1 || K == 2 || K == 5 || K == 8, "pair<K> takes the direction with s = +1");
         constexpr int C = comp(K), W = wclass(K);
         R s1p, s1m, s2p, s2m;  // A_i +- V_i
-        if constexpr (C < 2) {
+        if constexpr (MRT) {
+            R V1, V2;
+            if constexpr (C < 2) {
+                V1 = fma(R(4), Q1[C], D1[C]);
+                V2 = fma(R(4), Q2[C], D2[C]);
+            } else {
+                V1 = C == 2 ? Qd1[0] + Qd1[1] : Qd1[0] - Qd1[1];
+                V2 = C == 2 ? Qd2[0] + Qd2[1] : Qd2[0] - Qd2[1];
+            }
+            s1p = A1[W] + V1;
+            s1m = A1[W] - V1;
+            s2p = A2[W] + V2;
+            s2m = A2[W] - V2;
+        } else if constexpr (C < 2) {
             s1p = fma(R(4), Q1[C], A1[W]);
             s1m = fma(R(-4), Q1[C], A1[W]);
             s2p = fma(R(4), Q2[C], A2[W]);
@@ -489,6 +573,11 @@ __device__ __forceinline__ void mrt_relax(const R v[9], const R veq[9], const R 
     }
 }
 
+// The moment-space form with the dense transforms, which FP32 arithmetic keeps:
+// in FP32 the pairwise form carries the rounding of the BGK constants (1 -
+// 1/tau_g against rho w/tau_g) into the momentum, and after 255 steps of a
+// 235x790 lattice the velocity was 1.5e-5 off the FP64 one against 4.6e-6 here
+// (for 1.16 times the speed); 16-bit storage would round differently.
 // Per-node inputs of the MRT update: equilibria (Eqs. 2a, 2b) and the source
 // terms of Eqs. 11a, 11b without their (1 - 1/(2 tau)) factors; the F_a part of
 // Eq. 11b is added after the relaxation.

@@ -312,7 +312,7 @@ __device__ __forceinline__ void interior_tile_ip(S* f, CuT<S>* __restrict__ cu, 
         if constexpr (kPre) {
             if (!PREFETCH) load_all_f();
         }
-        CollideOf<MRT, R, UNI> col;
+        CollideOf<S, MRT, R, UNI> col;
         col.build(P, m, h, c1ux - cp[0], c1uy - cp[1], c2ux - cp[2], c2uy - cp[3]);
         collide_all_inplace<S, R>(col, gv,
             [&](auto kc, R& f1k, R& f2k) {
@@ -422,7 +422,7 @@ __device__ __forceinline__ void wall_node_ip(S* f, CuT<S>* __restrict__ cu, cons
         cu[1 * PL + o] = CuT<S>(c1uy);
         cu[2 * PL + o] = CuT<S>(c2ux);
         cu[3 * PL + o] = CuT<S>(c2uy);
-        CollideOf<MRT, R> col;
+        CollideOf<S, MRT, R> col;
         col.build(P, m, h, d1x, d1y, d2x, d2y);
         collide_all_inplace<S, R>(col, gv,
             [&](auto kc, R& f1k, R& f2k) {
@@ -456,7 +456,7 @@ __device__ __forceinline__ void wall_node_ip(S* f, CuT<S>* __restrict__ cu, cons
         cu[1 * PL + o] = CuT<S>(0);
         cu[2 * PL + o] = CuT<S>(c2ux);
         cu[3 * PL + o] = CuT<S>(0);
-        CollideOf<MRT, R> col;
+        CollideOf<S, MRT, R> col;
         col.build(P, m, h, d1x, d1y, d2x, d2y);
         // Eq. 51: f(x_u) = f^eq(x_u) + [f(x_f) - f^eq(x_f)], for f^1, f^2 and g
         R gu[9], f1u[9], f2u[9];

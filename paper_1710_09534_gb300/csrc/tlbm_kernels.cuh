@@ -311,8 +311,9 @@ __device__ __forceinline__ void rest_add(float hi, float lo, float d, float& nhi
 // storage, 0 otherwise).  With 16-bit storage the outputs are encoded once
 // here and handed to `store` as Bits16; the rest pair sees the decoded
 // (stored) values, so the mass bookkeeping is unchanged.
-template <typename S, typename R, int SE = 0, bool UNI, typename Load, typename LoadLo, typename St, typename StLo>
-__device__ __forceinline__ void collide_all(const Collider<R, UNI>& col, const R gv[9], Load load, LoadLo load_lo,
+template <typename S, typename R, int SE = 0, bool UNI, bool MRT, typename Load, typename LoadLo, typename St,
+          typename StLo>
+__device__ __forceinline__ void collide_all(Collider<R, UNI, MRT>& col, const R gv[9], Load load, LoadLo load_lo,
                                             St store, StLo store_lo)
 {
     constexpr bool ff = Store<S>::kLo;
@@ -327,6 +328,20 @@ __device__ __forceinline__ void collide_all(const Collider<R, UNI>& col, const R
             return Bits16{0};
         }
     };
+    if constexpr (MRT) {
+        col.moments_of_g(gv);
+        R p1[4], p2[4];  // f_k - f_k-bar of the four opposite pairs
+        static_for<0, 4>([&](auto pc) {
+            constexpr int I = decltype(pc)::value, K = pair_dir(I), KB = opp(K);
+            R a1, a2, b1, b2;
+            load(std::integral_constant<int, K>{}, a1, a2);
+            load(std::integral_constant<int, KB>{}, b1, b2);
+            p1[I] = a1 - b1;
+            p2[I] = a2 - b2;
+        });
+        col.flux_of_f(p1[0] + (p1[2] + p1[3]), p1[1] + (p1[2] - p1[3]), p2[0] + (p2[2] + p2[3]),
+                      p2[1] + (p2[2] - p2[3]));
+    }
     R d1 = R(0), d2 = R(0);  // sum_k (f_k - o'_k) over the moving directions
     // the directions go in opposite pairs (k, k-bar), which share most of
     // their arithmetic; both inputs of a pair are read before either output
@@ -433,17 +448,17 @@ __device__ __forceinline__ void collide_all(const MrtNode<R>& col, const R gv[9]
     });
 }
 
-// In-place form of the BGK collide_all: the post-collision populations of
+// In-place form of the pairwise collide_all: the post-collision populations of
 // direction k land in the location the input of direction k-bar came from
 // (and vice versa); collide_all already reads both inputs of an opposite pair
-// before it writes either output.
-template <typename S, typename R, bool UNI, typename Load, typename LoadLo, typename St, typename StLo>
-__device__ __forceinline__ void collide_all_inplace(const Collider<R, UNI>& col, const R gv[9], Load load,
+// before it writes either output (and MRT reads every pair before the first).
+template <typename S, typename R, bool UNI, bool MRT, typename Load, typename LoadLo, typename St, typename StLo>
+__device__ __forceinline__ void collide_all_inplace(Collider<R, UNI, MRT>& col, const R gv[9], Load load,
                                                     LoadLo load_lo, St store, StLo store_lo)
 {
     collide_all<S, R>(col, gv, load, load_lo, store, store_lo);
 }
-// MRT already reads all nine populations before writing any.
+// The dense MRT form reads all nine populations before writing any.
 template <typename S, typename R, typename Load, typename LoadLo, typename St, typename StLo>
 __device__ __forceinline__ void collide_all_inplace(const MrtNode<R>& col, const R gv[9], Load load, LoadLo load_lo,
                                                     St store, StLo store_lo)
@@ -452,9 +467,12 @@ __device__ __forceinline__ void collide_all_inplace(const MrtNode<R>& col, const
 }
 
 // Per-node collision data of the BGK (MRT = false) or MRT update; UNI: the
-// uniform-property form of the BGK update.
-template <bool MRT, typename R, bool UNI = false>
-using CollideOf = typename std::conditional<MRT, MrtNode<R>, Collider<R, UNI>>::type;
+// uniform-property form.  kDenseMrt: the moment-space form with dense
+// transforms (FP32 arithmetic).
+template <typename S, bool MRT>
+constexpr bool kDenseMrt = MRT && !std::is_same<S, double>::value;
+template <typename S, bool MRT, typename R, bool UNI = false>
+using CollideOf = typename std::conditional<kDenseMrt<S, MRT>, MrtNode<R>, Collider<R, UNI, MRT>>::type;
 
 // Destinations of the push from an interior node (x, y): the neighbouring
 // columns and rows, wrapped on a periodic axis (interior nodes never reach a
@@ -562,7 +580,7 @@ __host__ __device__ constexpr bool stash_hi(int k) { return k != 0 && pair_dir(s
 static_assert(stash_vec(0) == 4 && stash_vec(1) == 0 && stash_vec(3) == 0 && stash_vec(6) == 3 && stash_hi(6) &&
                   !stash_hi(8) && stash_hi(4) && !stash_hi(2),
               "stash slots follow the collision's direction pairs");
-// Used by the FP32-arithmetic BGK interior kernels (single lattices and
+// Used by the FP32-arithmetic interior kernels with pairwise collision (single lattices and
 // batches): 5% faster FP32 and 2% faster FP16 on the 2048^2 lattice than
 // re-reading the populations through the cache.
 #ifndef TLB_STASH32
@@ -883,7 +901,7 @@ __device__ __forceinline__ void interior_tile(const S* __restrict__ fA, S* __res
         cu[1 * PL + ou] = CuT<S>(c1uy);
         cu[2 * PL + ou] = CuT<S>(c2ux);
         cu[3 * PL + ou] = CuT<S>(c2uy);
-        CollideOf<MRT, R, UNI> col;
+        CollideOf<S, MRT, R, UNI> col;
         col.template build<SE>(P, m, h, c1ux - cp[0], c1uy - cp[1], c2ux - cp[2], c2uy - cp[3]);
         const PushOffsets po(g, xs, yu);
         const int su = (yu + 9) % 3;
@@ -931,7 +949,7 @@ k_step_interior(const S* __restrict__ fA, S* __restrict__ fB, CuT<S>* __restrict
                 const uint8_t* __restrict__ cls, Geo g, Prm<R> P, int rows)
 {
     __shared__ ColRings<R, BLOCK> sh;
-    if constexpr (kStashPops && std::is_same<R, float>::value && !MRT) {
+    if constexpr (kStashPops && std::is_same<R, float>::value && !kDenseMrt<S, MRT>) {
         __shared__ PopStash<R, BLOCK> stash;
         interior_tile<S, R, BLOCK, PREFETCH, MRT, UNI, true>(fA, fB, cu, cls, g, P, blockIdx.x, blockIdx.y, rows, sh,
                                                             &stash);
@@ -1133,7 +1151,7 @@ __device__ __forceinline__ void wall_node(const S* __restrict__ fA, S* __restric
         cu[1 * PL + o] = CuT<S>(c1uy);
         cu[2 * PL + o] = CuT<S>(c2ux);
         cu[3 * PL + o] = CuT<S>(c2uy);
-        CollideOf<MRT, R> col;
+        CollideOf<S, MRT, R> col;
         col.build(P, m, h, d1x, d1y, d2x, d2y);
         collide_all<S, R>(col, gv,
             [&](auto kc, R& f1k, R& f2k) {
@@ -1174,7 +1192,7 @@ __device__ __forceinline__ void wall_node(const S* __restrict__ fA, S* __restric
         cu[1 * PL + o] = CuT<S>(0);
         cu[2 * PL + o] = CuT<S>(c2ux);
         cu[3 * PL + o] = CuT<S>(0);
-        CollideOf<MRT, R> col;
+        CollideOf<S, MRT, R> col;
         col.build(P, m, h, d1x, d1y, d2x, d2y);
         // Eq. 51: f(x_u) = f^eq(x_u) + [f(x_f) - f^eq(x_f)], for f^1, f^2 and g
         R gu[9], f1u[9], f2u[9];

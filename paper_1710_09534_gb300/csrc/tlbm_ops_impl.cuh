@@ -21,15 +21,14 @@ inline Prm<R> cast_prm(const Prm<double>& d)
         r.eta[i] = R(d.eta[i]);
         r.inv_tau[i] = R(d.inv_tau[i]);
         r.omt[i] = R(d.omt[i]);
-        r.src_f[i] = R(d.src_f[i]);
         r.e0[i] = R(d.e0[i]);
+        r.rate[i] = R(d.rate[i]);
+        r.kj[i] = R(d.kj[i]);
         r.drho[i] = R(d.drho[i]);
         r.dnu[i] = R(d.dnu[i]);
         r.aM[i] = R(d.aM[i]);
         for (int c = 0; c < 2; c++) {
             r.aw[i][c] = R(d.aw[i][c]);
-            r.bw[i][c] = R(d.bw[i][c]);
-            r.sw[i][c] = R(d.sw[i][c]);
         }
     }
     r.lamT = R(d.lamT);
@@ -65,7 +64,6 @@ inline Prm<R> cast_prm(const Prm<double>& d)
         r.K34l6[i] = R(d.K34l6[i]);
         r.drho12[i] = R(d.drho12[i]);
         r.aM6[i] = R(d.aM6[i]);
-        r.k3tau[i] = R(d.k3tau[i]);
         r.kq[i] = R(d.kq[i]);
         r.ks[i] = R(d.ks[i]);
         r.K3w3[i] = R(d.K3w3[i]);
