@@ -165,7 +165,7 @@ int tlb_create_lattice(int nx, int ny, int precision, const int32_t edges[4],
  * A solid node is never updated; its fluid neighbours use the wetting ghost
  * rule (Eq. 42, wetting solids) or the symmetric rule (neutral solids) and
  * bounce back on links into it (Eq. 44).  With a lid, rows ny-2 and ny-1 must
- * be fluid.  Builds the node classes and the compacted near-wall list on the
+ * be fluid.  Builds the node classes and the near-wall work list on the
  * host and uploads them (synchronizes the stream).  Must be followed by
  * tlb_set_fields before the next step. */
 int tlb_set_geometry(tlb_lattice *lat, const uint8_t *host_mask);
@@ -193,9 +193,11 @@ int tlb_set_fields_device(tlb_lattice *lat, const double *c1, const double *c2,
                           const double *ux, const double *uy, const double *p);
 
 /* Advance n >= 0 time steps, asynchronously on the stream: per step one fused
- * interior kernel and one near-wall kernel (in-place lattices: the
+ * interior kernel and one near-wall kernel, or one kernel over all nodes where
+ * that is faster (two-buffer lattices up to about 3.0, 1.4 and 0.75 million
+ * nodes in FP64, FP32 and 16-bit storage); in-place lattices: the
  * order-parameter pass, the interior kernel, the lid row if any, the
- * near-wall kernel, and after a last even step the in-place streaming).  The
+ * near-wall kernel, and after a last even step the in-place streaming.  The
  * near-wall launches run on a stream the lattice owns, ordered after the
  * step's earlier work and joined back into the caller's stream before the
  * step ends, so work the caller queues after tlb_step sees the whole step.
@@ -268,21 +270,24 @@ int tlb_theta12_from(double sigma12, double sigma13, double sigma23, double thet
  * starts recording events around the fused interior launch and the
  * near-wall launch of every step (and clears the totals); enable = 0 stops.
  * tlb_profile_read synchronizes and returns the summed device milliseconds
- * ms[0] (interior kernel), ms[1] (near-wall kernel) and the launch counts. */
+ * ms[0] (interior kernel), ms[1] (near-wall kernel) and the launch counts; a
+ * lattice stepped by one kernel over all nodes reports it as the interior one,
+ * with no near-wall launch. */
 int tlb_profile(tlb_lattice *lat, int enable);
 int tlb_profile_read(tlb_lattice *lat, double ms[2], int64_t launches[2]);
 
-/* Number of nodes in the near-wall list (handled by the near-wall kernel). */
+/* Number of near-wall nodes (handled by the near-wall kernel). */
 int64_t tlb_wall_nodes(tlb_lattice *lat);
 
 /* ---- Batches: many lattices advanced together -------------------------
- * A batch steps all its member lattices in lockstep: per step, one
- * persistent kernel whose blocks take (member, strip, segment) tiles of the
- * fused interior update from a shared counter and, concurrently on a stream
- * the batch owns, one loop over all the members' near-wall nodes (same
- * per-node arithmetic as tlb_step, so a member's result does not depend on
- * the rest of the batch).  Pairs of steps run as one captured CUDA graph on
- * the batch's stream (the side stream's launches are captured with it).
+ * A batch steps all its member lattices in lockstep, one launch per step: a
+ * persistent kernel whose blocks take the members' near-wall tiles and (member,
+ * strip, segment) tiles of the fused interior update from a shared counter, or,
+ * when the members together have no more nodes than a lattice that tlb_step
+ * steps by one kernel, one block per tile of that kernel (same per-node
+ * arithmetic as tlb_step, so a member's result does not depend on the rest of
+ * the batch).  Pairs of steps run as one captured CUDA graph on the batch's
+ * stream.
  * In-place lattices (TLB_INPLACE) cannot be members.  Members keep their
  * own workspaces; the batch workspace holds the device descriptors and work
  * lists.  Not in the paper: it serves many independent simulations.
@@ -296,11 +301,13 @@ int64_t tlb_wall_nodes(tlb_lattice *lat);
  * tlb_batch_remove synchronizes the batch stream.  tlb_batch_step advances
  * every member n steps, asynchronously.  tlb_batch_config sets the tile shape
  * (threads 64 or 128; row segments rows_small for members with ny <=
- * small_ny, rows_large otherwise).
+ * small_ny, rows_large otherwise); batches stepped by one block per tile have
+ * one shape only and keep the setting for when they grow.
  *
  * tlb_batch_tune times 8 candidate shapes on the batch's own members,
  * trial_steps + 2 trial steps each, keeps the fastest and reports {threads,
- * rows_small, rows_large, small_ny} and its time per step.  It leaves every
+ * rows_small, rows_large, small_ny} and its time per step (one block per tile:
+ * times and reports the current setting).  It leaves every
  * member's state as it was: each trial step reads the members' current
  * distributions and writes their spare buffer without making it current, and
  * the c_i u planes of Eq. 19 (the only state a step updates in place) are

@@ -125,7 +125,8 @@ int host_site(const tlb_lattice* L, int x, int y, int64_t* idx)
     return tlb::ST_FLUID;
 }
 
-// Node classes and the near-wall list from the host mask; uploads both.
+// Node classes and the near-wall tiles (in place: nodes) from the host mask;
+// uploads both.
 int build_geometry(tlb_lattice* L)
 {
     const int nx = L->nx, ny = L->ny, pitch = L->lay.pitch;
@@ -150,6 +151,8 @@ int build_geometry(tlb_lattice* L)
     }
     L->nlist = (int64_t)list.size();
     L->hlist = list;
+    if (!L->lay.inplace) list = tlb::wall_tiles(list, L->geo, tlb::kWallTY);
+    L->nwork = (int64_t)list.size();
     TLB_CUDA(cudaMemcpyAsync(L->ws + L->lay.cls, L->cls.data(), L->cls.size(), cudaMemcpyHostToDevice,
                              L->stream));
     if (!list.empty())
@@ -158,6 +161,9 @@ int build_geometry(tlb_lattice* L)
     TLB_CUDA(cudaStreamSynchronize(L->stream));
     return TLB_OK;
 }
+
+// Whether a step of this lattice is one launch over all its nodes.
+bool one_launch(const tlb_lattice* L) { return !L->lay.inplace && L->ops->use_tile(L->n()); }
 
 constexpr int kProfSlots = 512;
 
@@ -175,7 +181,7 @@ int prof_fold(tlb_lattice* L)
         L->prof_ms[0] += a;
         L->prof_ms[1] += b;
         L->prof_n[0] += 1;
-        L->prof_n[1] += L->nlist > 0 ? 1 : 0;
+        L->prof_n[1] += L->nlist > 0 && !one_launch(L) ? 1 : 0;
     }
     L->ev_used = 0;
     return TLB_OK;
@@ -184,8 +190,9 @@ int prof_fold(tlb_lattice* L)
 // One step's launches: `interior` on the lattice's stream and `wall` on the
 // side stream between a fork after `pre` (work both depend on) and a join,
 // then `post` on the lattice's stream; with profiling, events around both.
+// two: whether the step has a near-wall launch.
 template <typename Pre, typename Interior, typename Wall, typename Post>
-int step_launches(tlb_lattice* L, Pre pre, Interior interior, Wall wall, Post post)
+int step_launches(tlb_lattice* L, bool two, Pre pre, Interior interior, Wall wall, Post post)
 {
     int rc;
     cudaEvent_t* ev = nullptr;
@@ -195,7 +202,6 @@ int step_launches(tlb_lattice* L, Pre pre, Interior interior, Wall wall, Post po
         TLB_CUDA(cudaEventRecord(ev[0], L->stream));
     }
     TLB_CUDA(pre());
-    const bool two = L->nlist > 0;
     // the near-wall launch goes first, so that its few blocks are resident
     // before the interior grid takes the SMs
     if (two) {
@@ -566,7 +572,7 @@ static int step_inplace(tlb_lattice* L, int64_t n)
     for (int64_t s = 0; s < n; s++) {
         const int odd = (int)(s & 1);
         rc = step_launches(
-            L, [&] { return L->ops->csum_ip(L->bufA(), L->cpl(), L->dcls(), L->geo, odd, L->stream); },
+            L, L->nlist > 0, [&] { return L->ops->csum_ip(L->bufA(), L->cpl(), L->dcls(), L->geo, odd, L->stream); },
             [&] { return L->ops->interior_ip(L->bufA(), L->cu(), L->cpl(), L->dcls(), L->geo, L->prm, odd, L->stream); },
             [&](cudaStream_t ws) {
                 cudaError_t e = cudaSuccess;
@@ -594,12 +600,23 @@ int tlb_step(tlb_lattice* L, int64_t n)
     if (!L->have_params || !L->have_fields) return fail(TLB_ESTATE, "set_params and set_fields before step");
     if (L->batch) return fail(TLB_ESTATE, "lattice belongs to a batch: step the batch");
     if (L->lay.inplace) return step_inplace(L, n);
+    if (one_launch(L)) {
+        for (int64_t s = 0; s < n; s++) {
+            rc = step_launches(
+                L, false, [] { return cudaSuccess; },
+                [&] { return L->ops->tile(L->bufA(), L->bufB(), L->cu(), L->dcls(), L->geo, L->prm, L->stream); },
+                [](cudaStream_t) { return cudaSuccess; }, [] { return cudaSuccess; });
+            if (rc) return rc;
+            L->cur ^= 1;
+        }
+        return ok();
+    }
     for (int64_t s = 0; s < n; s++) {
         rc = step_launches(
-            L, [] { return cudaSuccess; },
+            L, L->nlist > 0, [] { return cudaSuccess; },
             [&] { return L->ops->interior(L->bufA(), L->bufB(), L->cu(), L->dcls(), L->geo, L->prm, L->stream); },
             [&](cudaStream_t ws) {
-                return L->ops->wall(L->bufA(), L->bufB(), L->cu(), L->dcls(), L->dlist(), (int)L->nlist, L->geo,
+                return L->ops->wall(L->bufA(), L->bufB(), L->cu(), L->dcls(), L->dlist(), (int)L->nwork, L->geo,
                                     L->prm, ws);
             },
             [] { return cudaSuccess; });
@@ -896,6 +913,19 @@ const char* tlb_last_error(void) { return g_err.c_str(); }
 }  // extern "C"
 
 namespace tlb {
+
+std::vector<uint32_t> wall_tiles(const std::vector<uint32_t>& list, const Geo& g, int ty)
+{
+    const int shift = tile_shift(g.edge[3] == EDGE_LID, g.ny, ty);
+    const int cols = (g.nx + 31) / 32, rows = (g.ny + shift + ty - 1) / ty;
+    std::vector<uint8_t> has((size_t)cols * rows, 0);
+    for (uint32_t n : list) has[(size_t)(((n >> 16) + shift) / ty) * cols + (n & 0xffffu) / 32] = 1;
+    std::vector<uint32_t> tiles;
+    for (int r = 0; r < rows; r++)
+        for (int c = 0; c < cols; c++)
+            if (has[(size_t)r * cols + c]) tiles.push_back(((uint32_t)r << 16) | (uint32_t)c);
+    return tiles;
+}
 
 int lattice_view(tlb_lattice* L, LatticeView* v)
 {

@@ -70,15 +70,11 @@ struct tlb_batch {
     int rows_small = 16, rows_large = 16, small_ny = 128;
     bool dirty = true;
     int64_t n_tiles = 0, n_wall = 0;
-    int grid_interior = 0, grid_wall = 0;
+    bool tile = false;            // the members together are small enough for one-tile blocks (k_batch_tile)
+    int grid = 0;
     cudaGraphExec_t graph = nullptr;
-    int graph_variant = -1;
+    int graph_variant = -1, graph_grid = 0;
     const tlb::Ops* graph_ops = nullptr;
-    // the near-wall loop of a step runs on `side`, concurrently with the
-    // interior tile queue (disjoint writes, one state read), between `fork`
-    // and `join` (captured into the graph like the launches)
-    cudaStream_t side = nullptr;
-    cudaEvent_t fork = nullptr, join = nullptr;
 };
 
 namespace {
@@ -110,7 +106,12 @@ int rebuild(tlb_batch* B)
                      [&](int a, int b) { return B->members[a]->n() > B->members[b]->n(); });
     std::vector<tlb::TileItem> tiles;
     std::vector<tlb::WallItem> walls;
-    const int tx = (B->variant == 0 ? 64 : 128) - 4;
+    int64_t wall_nodes = 0;
+    int64_t nodes = 0;
+    for (const tlb_lattice* L : B->members) nodes += L->n();
+    B->tile = B->ops->use_tile(nodes);
+    // columns and rows of an item
+    const int tx = B->tile ? 64 : (B->variant == 0 ? 64 : 128) - 4;
     for (size_t i = 0; i < B->members.size(); i++) {
         tlb_lattice* L = B->members[i];
         B->ops->fill_desc(descs.data() + ds * i, L->bufA(), L->bufB(), L->cu(), L->dcls(), L->geo, L->prm,
@@ -119,16 +120,20 @@ int rebuild(tlb_batch* B)
     }
     for (int i : order) {
         tlb_lattice* L = B->members[i];
-        const int rows = rows_for(B, L);
+        const int rows = B->tile ? tlb::kBatchTY : rows_for(B, L);
+        // (with a lid row the tiles may start a row lower: as many rows of tiles)
         const int nbx = (L->nx + tx - 1) / tx, nby = (L->ny + rows - 1) / rows;
         for (int by = 0; by < nby; by++)
             for (int bx = 0; bx < nbx; bx++) tiles.push_back({i, bx, by});
-        for (uint32_t p : L->hlist) walls.push_back({i, p});
+        if (!B->tile)
+            for (uint32_t p : tlb::wall_tiles(L->hlist, L->geo, B->variant == 0 ? 2 : 4)) walls.push_back({i, p});
+        wall_nodes += L->nlist;
     }
-    if ((int64_t)tiles.size() > B->max_tiles || (int64_t)walls.size() > B->max_wall)
-        return err(TLB_ENOMEM, "batch needs %zu tiles and %zu wall nodes; capacity %lld and %lld", tiles.size(),
-                   walls.size(), (long long)B->max_tiles, (long long)B->max_wall);
-    tlb::BatchCounters c{(int)tiles.size(), (int)walls.size(), {0, 0}};
+    // (a near-wall tile holds at least one near-wall node)
+    if ((int64_t)tiles.size() > B->max_tiles || wall_nodes > B->max_wall)
+        return err(TLB_ENOMEM, "batch needs %zu tiles and %lld wall nodes; capacity %lld and %lld", tiles.size(),
+                   (long long)wall_nodes, (long long)B->max_tiles, (long long)B->max_wall);
+    tlb::BatchCounters c{(int)tiles.size(), (int)walls.size(), 0, 0};
     if (!descs.empty())
         B_CUDA(cudaMemcpyAsync(B->ws + B->lay.desc, descs.data(), descs.size(), cudaMemcpyHostToDevice, B->stream));
     if (!tiles.empty())
@@ -144,28 +149,26 @@ int rebuild(tlb_batch* B)
     int sms = 0;
     B_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, B->device));
     const int per_sm = std::max(1, B->ops->batch_blocks_per_sm(B->variant));
-    B->grid_interior = sms * per_sm;
-    B->grid_wall = 2 * sms;
+    B->grid = B->tile ? 2 * (int)tiles.size() : sms * per_sm;
     B->dirty = false;
     return TLB_OK;
 }
 
+int step_variant(const tlb_batch* B) { return B->tile ? 2 : B->variant; }
+
 int launch_step(tlb_batch* B, int parity)
 {
-    B_CUDA(cudaEventRecord(B->fork, B->stream));
-    B_CUDA(cudaStreamWaitEvent(B->side, B->fork, 0));
     B_CUDA(B->ops->batch_step(B->ws + B->lay.desc, B->ws + B->lay.tiles, B->ws + B->lay.walls, B->ws + B->lay.ctr,
-                              parity, B->variant, B->grid_interior, B->grid_wall, B->stream, B->side));
-    B_CUDA(cudaEventRecord(B->join, B->side));
-    B_CUDA(cudaStreamWaitEvent(B->stream, B->join, 0));
+                              parity, step_variant(B), B->grid, B->stream));
     return TLB_OK;
 }
 
-// Graph of one even and one odd step (valid for any membership: the counts
-// and descriptors live in device memory).
+// Graph of one even and one odd step (with the persistent kernel valid for any
+// membership: the counts and descriptors live in device memory).
 int ensure_graph(tlb_batch* B)
 {
-    if (B->graph && B->graph_variant == B->variant && B->graph_ops == B->ops) return TLB_OK;
+    if (B->graph && B->graph_variant == step_variant(B) && B->graph_grid == B->grid && B->graph_ops == B->ops)
+        return TLB_OK;
     if (B->graph) {
         cudaGraphExecDestroy(B->graph);
         B->graph = nullptr;
@@ -180,7 +183,8 @@ int ensure_graph(tlb_batch* B)
     const cudaError_t ei = cudaGraphInstantiate(&B->graph, g, 0);
     cudaGraphDestroy(g);
     if (ei != cudaSuccess) return err(TLB_ECUDA, "graph instantiate failed: %s", cudaGetErrorString(ei));
-    B->graph_variant = B->variant;
+    B->graph_variant = step_variant(B);
+    B->graph_grid = B->grid;
     B->graph_ops = B->ops;
     return TLB_OK;
 }
@@ -314,15 +318,6 @@ int tlb_batch_create(int precision, int max_lattices, int64_t max_tiles, int64_t
         delete B;
         return err(TLB_ECUDA, "no current device");
     }
-    cudaError_t e = cudaEventCreateWithFlags(&B->fork, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&B->join, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&B->side, cudaStreamNonBlocking);
-    if (e != cudaSuccess) {
-        if (B->fork) cudaEventDestroy(B->fork);
-        if (B->join) cudaEventDestroy(B->join);
-        delete B;
-        return err(TLB_ECUDA, "batch set-up failed: %s", cudaGetErrorString(e));
-    }
     *out = B;
     return tlb::clear_error();
 }
@@ -426,11 +421,17 @@ int tlb_batch_tune(tlb_batch* B, int trial_steps_n, void* dev_scratch, int64_t s
     double best = 1e30;
     int best_i = 0;
     rc = copy_cu(B, (char*)dev_scratch, true);
-    for (int i = 0; rc == TLB_OK && i < (int)(sizeof shapes / sizeof shapes[0]); i++) {
-        B->variant = shapes[i][0] == 64 ? 0 : 1;
-        B->rows_small = shapes[i][1];
-        B->rows_large = shapes[i][2];
-        B->small_ny = 128;
+    int64_t nodes = 0;
+    for (const tlb_lattice* L : B->members) nodes += L->n();
+    // (one-tile blocks have one shape: the current one is timed and kept)
+    const bool one = B->ops->use_tile(nodes);
+    const int current[3] = {B->variant == 0 ? 64 : 128, B->rows_small, B->rows_large};
+    const int (*cand)[3] = one ? &current : shapes;
+    for (int i = 0; rc == TLB_OK && i < (one ? 1 : (int)(sizeof shapes / sizeof shapes[0])); i++) {
+        B->variant = cand[i][0] == 64 ? 0 : 1;
+        B->rows_small = cand[i][1];
+        B->rows_large = cand[i][2];
+        B->small_ny = one ? saved[3] : 128;
         B->dirty = true;
         if ((rc = trial_steps(B, 2))) break;  // warm-up (also rebuilds the lists)
         cudaError_t ce = cudaEventRecord(e0, B->stream);
@@ -463,13 +464,13 @@ int tlb_batch_tune(tlb_batch* B, int trial_steps_n, void* dev_scratch, int64_t s
         return rc ? rc : rc_restore;
     }
     if (es != cudaSuccess) return err(TLB_ECUDA, "batch stream: %s", cudaGetErrorString(es));
-    B->variant = shapes[best_i][0] == 64 ? 0 : 1;
-    B->rows_small = shapes[best_i][1];
-    B->rows_large = shapes[best_i][2];
+    B->variant = cand[best_i][0] == 64 ? 0 : 1;
+    B->rows_small = cand[best_i][1];
+    B->rows_large = cand[best_i][2];
     if (out_config) {
-        out_config[0] = shapes[best_i][0];
-        out_config[1] = shapes[best_i][1];
-        out_config[2] = shapes[best_i][2];
+        out_config[0] = cand[best_i][0];
+        out_config[1] = cand[best_i][1];
+        out_config[2] = cand[best_i][2];
         out_config[3] = B->small_ny;
     }
     if (out_ms_per_step) *out_ms_per_step = best;
@@ -483,9 +484,6 @@ void tlb_batch_destroy(tlb_batch* B)
     cudaStreamSynchronize(B->stream);
     for (tlb_lattice* L : B->members) L->batch = nullptr;
     if (B->graph) cudaGraphExecDestroy(B->graph);
-    cudaEventDestroy(B->fork);
-    cudaEventDestroy(B->join);
-    cudaStreamDestroy(B->side);
     delete B;
 }
 

@@ -1,17 +1,20 @@
 // Batched execution: many lattices of different sizes advanced together.
 //
 // Each member lattice is described on the device by a LatDesc (its buffers,
-// geometry, parameters and row-segment length).  One step of the batch is
-//   k_batch_interior: a persistent kernel whose blocks take tiles (member,
-//                     strip, segment) from a shared counter until the tile
-//                     list is exhausted, running the same tile code as the
-//                     single-lattice fused kernel;
-//   k_batch_wall:     a grid-stride loop over the concatenated near-wall
-//                     lists of all members.
-// Tile and wall counts live in device memory, so one captured CUDA graph of a
-// pair of steps stays valid when the membership changes.
+// geometry, parameters and row-segment length).  One step of the batch is one
+// launch:
+//   k_batch_interior: a persistent kernel whose blocks take items from a shared
+//                     counter until the list is exhausted: first the members'
+//                     near-wall tiles (k_step_wall's code), then their interior
+//                     tiles (member, strip, segment), running the same tile
+//                     code as the single-lattice kernels;
+//   k_batch_tile:     for batches whose members together are small enough for
+//                     k_step_tile: two tiles of 32 x 8 nodes per item.
+// The item counts live in device memory, so one captured CUDA graph of a pair
+// of steps of k_batch_interior stays valid when the membership changes.
 #pragma once
 #include "tlbm_kernels.cuh"
+#include "tlbm_tile.cuh"
 
 namespace tlb {
 
@@ -31,65 +34,118 @@ struct TileItem {
 
 struct WallItem {
     int lat;
-    uint32_t packed;  // (y << 16) | x
+    uint32_t packed;  // (row << 16) | column of a near-wall tile of 32 x (threads / 32) nodes
 };
+
+constexpr int kBatchTY = 8;  // rows of a tile of k_batch_tile
 
 struct BatchCounters {
     int n_tiles, n_wall;
-    int next[2];  // tile counters of the two step parities (reset before each launch)
+    int next, done;  // items taken and blocks finished of the running launch (zero between launches)
 };
 
+// One near-wall tile of a member; a call of its own, so that its registers are
+// not the interior update's (inlined, FP64 spilled 40 words and FP16 100).
+template <typename S, typename R, int TY, bool MRT>
+__device__ __noinline__ void batch_wall_item(const LatDesc<R>* d, int parity, const Prm<R>& P, int bx, int by,
+                                             TileShared<R, TY>& sh)
+{
+    const Geo g = d->g;
+    tile_step<S, R, TY, MRT, false, true>((const S*)d->buf[parity], (S*)d->buf[parity ^ 1], (CuT<S>*)d->cu, d->cls, g, P,
+                                          bx * 32, by * TY - tile_shift(g.edge[3] == EDGE_LID, g.ny, TY), sh);
+}
+
+// The near-wall tiles go through the interior kernel's own queue, before the
+// interior tiles: as a launch of their own beside it they either waited for
+// the persistent blocks, which fill every register file, or kept some of them
+// from starting (32 lattices of 64..512 nodes a side, FP32, GB300: 109
+// -> 99 us per step).
 template <typename S, typename R, int BLOCK, bool PREFETCH, int MINB, bool MRT>
 __global__ void __launch_bounds__(BLOCK, MINB)
 k_batch_interior(const LatDesc<R>* __restrict__ descs, const TileItem* __restrict__ items,
-                 BatchCounters* __restrict__ ctr, int parity)
+                 const WallItem* __restrict__ walls, BatchCounters* __restrict__ ctr, int parity)
 {
-    __shared__ ColRings<R, BLOCK> sh;
+    constexpr int WTY = BLOCK / 32;
     constexpr bool kStash = kStashPops && std::is_same<R, float>::value && !kDenseMrt<S, MRT>;
-    __shared__ PopStash<R, kStash ? BLOCK : 1> stash;
+    struct March {
+        ColRings<R, BLOCK> rings;
+        PopStash<R, kStash ? BLOCK : 1> stash;
+    };
+    // an item is either kind, so its shared data share one place
+    constexpr size_t kBytes = sizeof(March) > sizeof(TileShared<R, WTY>) ? sizeof(March) : sizeof(TileShared<R, WTY>);
+    __shared__ __align__(16) unsigned char raw[kBytes];
+    March& sh = *reinterpret_cast<March*>(raw);
     __shared__ Prm<R> Ps;
     __shared__ int item_s;
     static_assert(sizeof(Prm<R>) % sizeof(R) == 0, "params are whole words");
     constexpr int kWords = (int)(sizeof(Prm<R>) / sizeof(R));
-    const int n = ctr->n_tiles;
+    const int nw = ctr->n_wall, n = nw + ctr->n_tiles;
+    // the state, and the counters, are those of the previous launch
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     for (;;) {
-        if (threadIdx.x == 0) item_s = atomicAdd(&ctr->next[parity], 1);
+        if (threadIdx.x == 0) item_s = atomicAdd(&ctr->next, 1);
         __syncthreads();
         const int it = item_s;
         if (it >= n) break;
-        const TileItem ti = items[it];
+        const bool wall = it < nw;
+        const TileItem ti = wall ? TileItem{walls[it].lat, (int)(walls[it].packed & 0xffffu), (int)(walls[it].packed >> 16)}
+                                 : items[it - nw];
         const LatDesc<R>* d = descs + ti.lat;
         for (int i = threadIdx.x; i < kWords; i += BLOCK)
             reinterpret_cast<R*>(&Ps)[i] = reinterpret_cast<const R*>(&d->P)[i];
         __syncthreads();
         const Geo g = d->g;
+        const S* fA = (const S*)d->buf[parity];
+        S* fB = (S*)d->buf[parity ^ 1];
+        CuT<S>* cu = (CuT<S>*)d->cu;
         // members with equal densities and viscosities take the uniform-property
         // update, as they do when stepped alone (the branch is uniform per tile)
-        auto* st = reinterpret_cast<PopStash<R, BLOCK>*>(&stash);  // used only when kStash
-        if (Ps.uni != R(0))
-            interior_tile<S, R, BLOCK, PREFETCH, MRT, true, kStash>((const S*)d->buf[parity], (S*)d->buf[parity ^ 1],
-                                                                    (CuT<S>*)d->cu, d->cls, g, Ps, ti.bx, ti.by,
-                                                                    d->rows, sh, st);
+        auto* st = reinterpret_cast<PopStash<R, BLOCK>*>(&sh.stash);  // used only when kStash
+        if (wall)
+            batch_wall_item<S, R, WTY, MRT>(d, parity, Ps, ti.bx, ti.by, *reinterpret_cast<TileShared<R, WTY>*>(raw));
+        else if (Ps.uni != R(0))
+            interior_tile<S, R, BLOCK, PREFETCH, MRT, true, kStash>(fA, fB, cu, d->cls, g, Ps, ti.bx, ti.by, d->rows,
+                                                                    sh.rings, st);
         else
-            interior_tile<S, R, BLOCK, PREFETCH, MRT, false, kStash>((const S*)d->buf[parity], (S*)d->buf[parity ^ 1],
-                                                                     (CuT<S>*)d->cu, d->cls, g, Ps, ti.bx, ti.by,
-                                                                     d->rows, sh, st);
-        __syncthreads();  // rings, parameters and item_s are reused by the next tile
+            interior_tile<S, R, BLOCK, PREFETCH, MRT, false, kStash>(fA, fB, cu, d->cls, g, Ps, ti.bx, ti.by, d->rows,
+                                                                     sh.rings, st);
+        __syncthreads();  // shared data, parameters and item_s are reused by the next item
+    }
+    // the last block leaves the counters as the next launch expects them
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(&ctr->done, 1) == (int)gridDim.x - 1) {
+            ctr->next = 0;
+            ctr->done = 0;
+        }
     }
 }
 
-template <typename S, typename R, bool MRT>
-__global__ void __launch_bounds__(128)
-k_batch_wall(const LatDesc<R>* __restrict__ descs, const WallItem* __restrict__ items,
-             const BatchCounters* __restrict__ ctr, int parity)
+// Blocks 2i, 2i + 1: the left and right tile of 32 x kBatchTY nodes of item i
+// (columns 64 bx .., rows kBatchTY by ..).
+template <typename S, typename R, int MINB, bool MRT>
+__global__ void __launch_bounds__(32 * kBatchTY, MINB)
+k_batch_tile(const LatDesc<R>* __restrict__ descs, const TileItem* __restrict__ items, int parity)
 {
-    const int n = ctr->n_wall;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const WallItem wi = items[i];
-        const LatDesc<R>* d = descs + wi.lat;
-        wall_node<S, R, MRT>((const S*)d->buf[parity], (S*)d->buf[parity ^ 1], (CuT<S>*)d->cu, d->cls, d->g, d->P,
-                        wi.packed);
-    }
+    __shared__ TileShared<R, kBatchTY> sh;
+    __shared__ Prm<R> Ps;
+    constexpr int kWords = (int)(sizeof(Prm<R>) / sizeof(R));
+    const TileItem ti = items[blockIdx.x >> 1];
+    const LatDesc<R>* d = descs + ti.lat;
+    const int x0 = ti.bx * 64 + (blockIdx.x & 1) * 32;
+    if (x0 >= d->g.nx) return;
+    for (int i = threadIdx.x; i < kWords; i += 32 * kBatchTY)
+        reinterpret_cast<R*>(&Ps)[i] = reinterpret_cast<const R*>(&d->P)[i];
+    __syncthreads();
+    const Geo g = d->g;
+    const S* fA = (const S*)d->buf[parity];
+    S* fB = (S*)d->buf[parity ^ 1];
+    const int y0 = ti.by * kBatchTY - tile_shift(g.edge[3] == EDGE_LID, g.ny, kBatchTY);
+    if (Ps.uni != R(0))
+        tile_step<S, R, kBatchTY, MRT, true, false>(fA, fB, (CuT<S>*)d->cu, d->cls, g, Ps, x0, y0, sh);
+    else
+        tile_step<S, R, kBatchTY, MRT, false, false>(fA, fB, (CuT<S>*)d->cu, d->cls, g, Ps, x0, y0, sh);
 }
 
 }  // namespace tlb

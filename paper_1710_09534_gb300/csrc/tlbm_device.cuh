@@ -39,6 +39,12 @@ struct Geo {
     long long plane;  // elements per plane = ny * pitch
 };
 
+// Rows of a near-wall tile (k_step_wall), and the rows by which the first tile
+// of height ty starts below row 0, so that a lid row never is the first row of
+// its tile (its window reaches three rows down).
+constexpr int kWallTY = 4;
+__host__ __device__ constexpr int tile_shift(bool lid, int ny, int ty) { return lid && ny % ty == 1 ? 1 : 0; }
+
 // Derived constants, computed on the host from tlb_params (index i: fluid
 // 1, 2; index c: direction class 0 = axis (w = 1/9), 1 = diagonal (w = 1/36)).
 template <typename R>
@@ -92,12 +98,12 @@ __device__ __forceinline__ int site_of(const Geo& g, const uint8_t* __restrict__
                                        long long& off)
 {
     if (x < 0 || x >= g.nx) {
-        const int e = g.edge[x < 0 ? 0 : 1];
+        const int e = x < 0 ? g.edge[0] : g.edge[1];
         if (e != EDGE_PERIODIC) return e == EDGE_WETTING ? ST_WET : ST_NEUTRAL;
         x = x < 0 ? x + g.nx : x - g.nx;
     }
     if (y < 0 || y >= g.ny) {
-        const int e = g.edge[y < 0 ? 2 : 3];
+        const int e = y < 0 ? g.edge[2] : g.edge[3];
         if (e == EDGE_LID) return ST_VOID;
         if (e != EDGE_PERIODIC) return e == EDGE_WETTING ? ST_WET : ST_NEUTRAL;
         y = y < 0 ? y + g.ny : y - g.ny;

@@ -40,8 +40,11 @@ struct tlb_lattice {
     bool have_params = false, have_fields = false;
     std::vector<uint8_t> mask;    // host copy of the solid mask
     std::vector<uint8_t> cls;     // host copy of the node classes (pitched)
-    int64_t nlist = 0;
-    std::vector<uint32_t> hlist;  // host copy of the near-wall list
+    int64_t nlist = 0;            // near-wall nodes
+    std::vector<uint32_t> hlist;  // the near-wall nodes (y << 16 | x)
+    // entries of the work list on the device: near-wall tiles, or with in-place
+    // streaming the near-wall nodes
+    int64_t nwork = 0;
     tlb_batch* batch = nullptr;   // batch this lattice belongs to, if any
     // optional per-kernel timing: per step, events around the interior launch
     // (on `stream`) and around the near-wall launch (on `side`)

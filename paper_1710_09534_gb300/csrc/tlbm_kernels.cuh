@@ -7,9 +7,7 @@
 //                    sums of the pre-collision f (push streaming keeps them
 //                    local), mu_1, mu_2 on the tile plus radius 1 in shared
 //                    memory, then the per-node update.
-//   k_step_wall      the same update for the compacted list of the other
-//                    fluid nodes, with the ghost rules of Eqs. 42-43,
-//                    bounce-back (Eq. 44) and the lid (Eqs. 51-53).
+//                    (the other fluid nodes: tlbm_tile.cuh)
 //   k_init, k_read_fields, k_mass_partials/k_mass_final
 #pragma once
 #include <type_traits>
@@ -1098,159 +1096,6 @@ struct PlaneFetch {
         b = c[PL + off];
     }
 };
-
-// Push of one post-collision triple along direction K from node (x, y) with
-// the wall rules: into a fluid node, back into slot K-bar on a solid link
-// (Eq. 44), or out through the lid.
-template <int K, typename S, typename V1, typename V2, typename VG>
-__device__ __forceinline__ void push_wall(const Geo& g, const uint8_t* __restrict__ cls, S* __restrict__ fB,
-                                          int x, int y, long long o, V1 o1, V2 o2, VG og)
-{
-    const long long PL = g.plane;
-    if constexpr (K == 0) {
-        st_pop(fB, 0, PL, o, o1);
-        st_pop(fB, 9, PL, o, o2);
-        st_pop(fB, 18, PL, o, og);
-        return;
-    }
-    long long d = 0;
-    const int s = site_of(g, cls, x + ex(K), y + ey(K), d);
-    if (fluidlike(s)) {
-        st_three(fB, K, PL, d, o1, o2, og);
-    } else if (s == ST_WET || s == ST_NEUTRAL) {
-        st_three(fB, opp(K), PL, o, o1, o2, og);
-    }
-}
-
-// ---------------------------------------------------------------------------
-// K2: near-wall and lid nodes from the compacted list.
-// ---------------------------------------------------------------------------
-template <typename S, typename R, bool MRT>
-__device__ __forceinline__ void wall_node(const S* __restrict__ fA, S* __restrict__ fB, CuT<S>* __restrict__ cu,
-                                          const uint8_t* __restrict__ cls, const Geo& g, const Prm<R>& P,
-                                          uint32_t packed)
-{
-    const int x = (int)(packed & 0xffffu), y = (int)(packed >> 16);
-    const long long PL = g.plane;
-    const long long o = (long long)y * g.pitch + x;
-    const int kind = cls[o] & CLS_KIND_MASK;
-    DistFetch<S, R> fetch{fA, PL};
-
-    if (kind == ST_FLUID) {
-        Macro<R> m;
-        window_macros(g, cls, P, x, y, fetch, m);
-        R gv[9];
-#pragma unroll
-        for (int k = 0; k < 9; k++) gv[k] = ld_pop<R>(fA, 18 + k, PL, o);
-        Hydro<R> h;
-        hydro_from_g(P, m, gv, h);
-        const R c1ux = m.c1 * h.ux, c1uy = m.c1 * h.uy, c2ux = m.c2 * h.ux, c2uy = m.c2 * h.uy;
-        const R d1x = c1ux - R(cu[0 * PL + o]), d1y = c1uy - R(cu[1 * PL + o]);
-        const R d2x = c2ux - R(cu[2 * PL + o]), d2y = c2uy - R(cu[3 * PL + o]);
-        cu[0 * PL + o] = CuT<S>(c1ux);
-        cu[1 * PL + o] = CuT<S>(c1uy);
-        cu[2 * PL + o] = CuT<S>(c2ux);
-        cu[3 * PL + o] = CuT<S>(c2uy);
-        CollideOf<S, MRT, R> col;
-        col.build(P, m, h, d1x, d1y, d2x, d2y);
-        collide_all<S, R>(col, gv,
-            [&](auto kc, R& f1k, R& f2k) {
-                constexpr int K = decltype(kc)::value;
-                f1k = ld_pop<R>(fA, K, PL, o);
-                f2k = ld_pop<R>(fA, 9 + K, PL, o);
-            },
-            [&](R& l1, R& l2) {
-                l1 = ld_lo<R>(fA, 0, PL, o);
-                l2 = ld_lo<R>(fA, 1, PL, o);
-            },
-            [&](auto kc, auto o1, auto o2, auto og) {
-                constexpr int K = decltype(kc)::value;
-                push_wall<K>(g, cls, fB, x, y, o, o1, o2, og);
-            },
-            [&](R l1, R l2) {
-                st_lo(fB, 0, PL, o, l1);
-                st_lo(fB, 1, PL, o, l2);
-            });
-    } else if (kind == ST_LID) {
-        // x_f is the node below; x_u takes its macros and gradients, u = (U0, 0)
-        const long long of = o - g.pitch;
-        Macro<R> m;
-        window_macros(g, cls, P, x, y - 1, fetch, m);
-        R gf[9];
-#pragma unroll
-        for (int k = 0; k < 9; k++) gf[k] = ld_pop<R>(fA, 18 + k, PL, of);
-        Hydro<R> hf;
-        hydro_from_g(P, m, gf, hf);
-        Hydro<R> h = hf;
-        h.ux = P.lid_u;
-        h.uy = R(0);
-        h.usq = P.lid_u * P.lid_u;
-        const R c1ux = m.c1 * h.ux, c2ux = m.c2 * h.ux;
-        const R d1x = c1ux - R(cu[0 * PL + o]), d1y = R(0) - R(cu[1 * PL + o]);
-        const R d2x = c2ux - R(cu[2 * PL + o]), d2y = R(0) - R(cu[3 * PL + o]);
-        cu[0 * PL + o] = CuT<S>(c1ux);
-        cu[1 * PL + o] = CuT<S>(0);
-        cu[2 * PL + o] = CuT<S>(c2ux);
-        cu[3 * PL + o] = CuT<S>(0);
-        CollideOf<S, MRT, R> col;
-        col.build(P, m, h, d1x, d1y, d2x, d2y);
-        // Eq. 51: f(x_u) = f^eq(x_u) + [f(x_f) - f^eq(x_f)], for f^1, f^2 and g
-        R gu[9], f1u[9], f2u[9];
-#pragma unroll
-        for (int k = 0; k < 9; k++) {
-            R e1u, e2u, egu, e1f, e2f, egf;
-            equilibria(k, P, m.c1, m.c2, m.mu1, m.mu2, m.rho, hf.p, h.ux, h.uy, e1u, e2u, egu);
-            equilibria(k, P, m.c1, m.c2, m.mu1, m.mu2, m.rho, hf.p, hf.ux, hf.uy, e1f, e2f, egf);
-            R ff1 = ld_pop<R>(fA, k, PL, of), ff2 = ld_pop<R>(fA, 9 + k, PL, of);
-            if constexpr (Store<S>::kLo) {
-                if (k == 0) {
-                    ff1 += ld_lo<R>(fA, 0, PL, of);
-                    ff2 += ld_lo<R>(fA, 1, PL, of);
-                }
-            }
-            f1u[k] = e1u + (ff1 - e1f);
-            f2u[k] = e2u + (ff2 - e2f);
-            gu[k] = egu + (gf[k] - egf);
-        }
-        collide_all<S, R>(col, gu,
-            [&](auto kc, R& f1k, R& f2k) {
-                constexpr int K = decltype(kc)::value;
-                f1k = f1u[K];
-                f2k = f2u[K];
-            },
-            [&](R& l1, R& l2) {
-                l1 = R(0);
-                l2 = R(0);
-            },
-            [&](auto kc, auto o1, auto o2, auto og) {
-                constexpr int K = decltype(kc)::value;
-                push_wall<K>(g, cls, fB, x, y, o, o1, o2, og);
-                // slots fed from beyond the lid receive nothing: keep them zero
-                if constexpr (ey(K) == -1) {
-                    long long dummy = 0;
-                    if (site_of(g, cls, x - ex(K), y + 1, dummy) == ST_VOID) {
-                        st_pop(fB, K, PL, o, R(0));
-                        st_pop(fB, 9 + K, PL, o, R(0));
-                        st_pop(fB, 18 + K, PL, o, R(0));
-                    }
-                }
-            },
-            [&](R l1, R l2) {
-                st_lo(fB, 0, PL, o, l1);
-                st_lo(fB, 1, PL, o, l2);
-            });
-    }
-}
-
-template <typename S, typename R, bool MRT>
-__global__ void __launch_bounds__(128)
-k_step_wall(const S* __restrict__ fA, S* __restrict__ fB, CuT<S>* __restrict__ cu,
-            const uint8_t* __restrict__ cls, const uint32_t* __restrict__ list, int nlist, Geo g, Prm<R> P)
-{
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= nlist) return;
-    wall_node<S, R, MRT>(fA, fB, cu, cls, g, P, list[t]);
-}
 
 // ---------------------------------------------------------------------------
 // Set-up: f = f^eq(c, mu(c), u), g = g^eq(p, rho(c), u), cu = c u, for rows

@@ -2,6 +2,7 @@
 #pragma once
 #include <cstddef>
 #include <cstdint>
+#include <vector>
 #include <cuda_runtime.h>
 #include "tlbm_device.cuh"
 
@@ -14,8 +15,13 @@ struct Ops {
     // one time step A -> B = interior tiles (fused kernel) + near-wall list
     cudaError_t (*interior)(const void* fA, void* fB, void* cu, const uint8_t* cls, const Geo& g,
                             const Prm<double>& P, cudaStream_t s);
-    cudaError_t (*wall)(const void* fA, void* fB, void* cu, const uint8_t* cls, const uint32_t* list,
-                        int nlist, const Geo& g, const Prm<double>& P, cudaStream_t s);
+    // (near-wall tiles, see k_step_wall)
+    cudaError_t (*wall)(const void* fA, void* fB, void* cu, const uint8_t* cls, const uint32_t* tiles,
+                        int ntiles, const Geo& g, const Prm<double>& P, cudaStream_t s);
+    // the same step in one launch (k_step_tile), for lattices (or batches) of few enough nodes (use_tile)
+    cudaError_t (*tile)(const void* fA, void* fB, void* cu, const uint8_t* cls, const Geo& g, const Prm<double>& P,
+                        cudaStream_t s);
+    bool (*use_tile)(long long nodes);
     cudaError_t (*init)(void* fA, void* cu, const uint8_t* cls, const double* c1, const double* c2,
                         const double* ux, const double* uy, const double* p, const Geo& g,
                         const Prm<double>& P, cudaStream_t s);
@@ -29,11 +35,11 @@ struct Ops {
     // selected by comps (FP64), into *out
     cudaError_t (*film)(const void* fA, const uint8_t* cls, int x, int y_top, int comps, double* out, const Geo& g,
                         cudaStream_t s);
-    // batched step: persistent interior kernel (variant 0: 64-thread blocks,
-    // 1: 128-thread blocks) over the tile list on s, the near-wall loop on ws
-    // (the caller orders ws after the previous step and s's next step after ws)
+    // batched step: `grid` blocks of the persistent kernel (variant 0: 64-thread
+    // blocks, 1: 128-thread blocks) over the near-wall and interior items, or
+    // (variant 2) two blocks of k_batch_tile for each item of `tiles`
     cudaError_t (*batch_step)(const void* descs, const void* tiles, const void* walls, void* ctr, int parity,
-                              int variant, int grid_interior, int grid_wall, cudaStream_t s, cudaStream_t ws);
+                              int variant, int grid, cudaStream_t s);
     // resident blocks per SM of the persistent interior kernel of a variant
     int (*batch_blocks_per_sm)(int variant);
     size_t desc_size;  // bytes of one device lattice descriptor
@@ -66,6 +72,10 @@ struct Ops {
 inline size_t elem_for(int precision) { return precision == 0 ? 8 : (precision == 1 ? 4 : 2); }
 inline int ndist_for(int precision) { return precision == 0 ? 27 : (precision == 1 ? 29 : 33); }
 inline size_t cu_elem_for(int precision) { return precision == 0 ? 8 : 4; }
+
+// Tiles of 32 x ty nodes (row << 16 | column, in order) that hold any of the
+// near-wall nodes `list` (y << 16 | x); k_step_wall: ty = kWallTY.
+std::vector<uint32_t> wall_tiles(const std::vector<uint32_t>& list, const Geo& g, int ty);
 
 const Ops& ops_f64();
 const Ops& ops_f32();

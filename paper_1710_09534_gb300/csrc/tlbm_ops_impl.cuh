@@ -4,6 +4,7 @@
 #include "tlbm_inplace.cuh"
 #include "tlbm_kernels.cuh"
 #include "tlbm_ops.h"
+#include "tlbm_tile.cuh"
 
 namespace tlb {
 
@@ -150,14 +151,74 @@ struct OpsImpl {
         }
         return cudaGetLastError();
     }
-    static cudaError_t wall(const void* fA, void* fB, void* cu, const uint8_t* cls, const uint32_t* list,
-                            int nlist, const Geo& g, const Prm<double>& Pd, cudaStream_t s)
+    static cudaError_t wall(const void* fA, void* fB, void* cu, const uint8_t* cls, const uint32_t* tiles,
+                            int ntiles, const Geo& g, const Prm<double>& Pd, cudaStream_t s)
     {
         const Prm<R> P = cast_prm<R>(Pd);
-        if (nlist > 0)
-            k_step_wall<S, R, MRT><<<(nlist + 127) / 128, 128, 0, s>>>((const S*)fA, (S*)fB, (CuT<S>*)cu, cls, list,
-                                                                   nlist, g, P);
+        if (ntiles > 0)
+            k_step_wall<S, R, MRT><<<ntiles, 32 * kWallTY, 0, s>>>((const S*)fA, (S*)fB, (CuT<S>*)cu, cls, tiles, g, P,
+                                                                   tile_shift(g.edge[3] == EDGE_LID, g.ny, kWallTY));
         return cudaGetLastError();
+    }
+    // A launch whose blocks may become resident while the launch before it in
+    // the stream finishes (the kernel waits for it: griddepcontrol.wait).
+    template <typename K, typename... A>
+    static cudaError_t launch_dependent(K k, dim3 grid, int threads, cudaStream_t s, A... args)
+    {
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at.val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = grid;
+        cfg.blockDim = dim3(threads);
+        cfg.stream = s;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, k, args...);
+    }
+    template <int TY, int MB>
+    static cudaError_t launch_tile(const void* fA, void* fB, void* cu, const uint8_t* cls, const Geo& g,
+                                   const Prm<double>& Pd, cudaStream_t s)
+    {
+        const Prm<R> P = cast_prm<R>(Pd);
+        const int shift = tile_shift(g.edge[3] == EDGE_LID, g.ny, TY);
+        const dim3 grid((g.nx + 31) / 32, (g.ny + shift + TY - 1) / TY);
+        auto* k = Pd.uni != 0.0 ? &k_step_tile<S, R, TY, MB, MRT, true> : &k_step_tile<S, R, TY, MB, MRT, false>;
+        return launch_dependent(k, grid, 32 * TY, s, (const S*)fA, (S*)fB, (CuT<S>*)cu, cls, g, P, shift);
+    }
+    // Tile height and resident blocks, GB300, us per step (4 x 2: TY = 4 at 2
+    // blocks per SM, and so on):
+    //   FP64 (bound by the FP64 unit, so by the busiest SM): short tiles while
+    //     they spread over more SMs: 128x64 16.5 (4 x 2), 23.8 (8 x 2); 250x150
+    //     26.5, 27.5; 240x280 55.9, 56.1; from about 4 short tiles per SM on, the
+    //     smaller frame: 512x512 150, 132; 1024x1024 550, 494.
+    //   FP32 and 16-bit storage: TY = 8; a third block per SM (80 registers)
+    //     pays once the grid exceeds 4 tiles per SM: FP32 240x280 5.8 (8 x 2),
+    //     7.4 (8 x 3); 512x256 9.7, 10.2; 512x512 16.2, 14.0; 1024x1024 69.5, 64.8.
+    static cudaError_t tile(const void* fA, void* fB, void* cu, const uint8_t* cls, const Geo& g,
+                            const Prm<double>& Pd, cudaStream_t s)
+    {
+        const long long few = 4LL * sm_count(), strips = (g.nx + 31) / 32;
+        if constexpr (std::is_same<R, double>::value) {
+            if (strips * ((g.ny + 3) / 4) <= few) return launch_tile<4, 2>(fA, fB, cu, cls, g, Pd, s);
+            return launch_tile<8, 2>(fA, fB, cu, cls, g, Pd, s);
+        } else {
+            if (strips * ((g.ny + 7) / 8) <= few) return launch_tile<8, 2>(fA, fB, cu, cls, g, Pd, s);
+            return launch_tile<8, 3>(fA, fB, cu, cls, g, Pd, s);
+        }
+    }
+    // One launch per step up to these sizes; beyond them the state no longer
+    // stays in L2 (FP32, 16-bit: the marching kernel's loads one row ahead cover
+    // more of the memory latency) or the near-wall launch is hidden (FP64).
+    // GB300, us per step, marching and near-wall kernels against this one: FP64
+    // 128x64 45.2, 16.5; 512x256 142, 102; 1024x1024 565, 494; 1024x2048 1339,
+    // 1190; 2048x2048 1940, 1938.  FP32 128x64 13.5, 3.7; 512x256 20.6, 9.7;
+    // 1024x1024 68.2, 64.8; 1200x1100 91.4, 88.0; 1024x2048 114, 127.  FP16
+    // 128x64 12.6, 3.9; 512x256 22.1, 10.2; 512x1024 31.7, 26.4; 1024x1024 48.2,
+    // 53.8.
+    static bool use_tile(long long nodes)
+    {
+        return nodes <= (std::is_same<S, double>::value ? 3000000 : std::is_same<S, float>::value ? 1400000 : 750000);
     }
     static cudaError_t init(void* fA, void* cu, const uint8_t* cls, const double* c1, const double* c2,
                             const double* ux, const double* uy, const double* p, const Geo& g,
@@ -199,20 +260,19 @@ struct OpsImpl {
     // the two block shapes the batch tuner chooses between
     static constexpr int kMinB64 = std::is_same<R, float>::value ? 8 : 6;
     static cudaError_t batch_step(const void* descs, const void* tiles, const void* walls, void* ctr, int parity,
-                                  int variant, int grid_interior, int grid_wall, cudaStream_t s, cudaStream_t ws)
+                                  int variant, int grid, cudaStream_t s)
     {
+        const LatDesc<R>* d = (const LatDesc<R>*)descs;
+        const TileItem* ti = (const TileItem*)tiles;
+        const WallItem* wi = (const WallItem*)walls;
         BatchCounters* c = (BatchCounters*)ctr;
-        cudaError_t e = cudaMemsetAsync(&c->next[parity], 0, sizeof(int), s);
-        if (e != cudaSuccess) return e;
+        if (variant == 2)
+            return launch_dependent(&k_batch_tile<S, R, kMinBBatchTile, MRT>, dim3(grid), 32 * kBatchTY, s, d, ti, parity);
         if (variant == 0)
-            k_batch_interior<S, R, 64, PREFETCH, kMinB64, MRT><<<grid_interior, 64, 0, s>>>(
-                (const LatDesc<R>*)descs, (const TileItem*)tiles, c, parity);
-        else
-            k_batch_interior<S, R, 128, PREFETCH, MINB, MRT><<<grid_interior, 128, 0, s>>>(
-                (const LatDesc<R>*)descs, (const TileItem*)tiles, c, parity);
-        k_batch_wall<S, R, MRT><<<grid_wall, 128, 0, ws>>>((const LatDesc<R>*)descs, (const WallItem*)walls, c, parity);
-        return cudaGetLastError();
+            return launch_dependent(&k_batch_interior<S, R, 64, PREFETCH, kMinB64, MRT>, dim3(grid), 64, s, d, ti, wi, c, parity);
+        return launch_dependent(&k_batch_interior<S, R, 128, PREFETCH, MINB, MRT>, dim3(grid), 128, s, d, ti, wi, c, parity);
     }
+    static constexpr int kMinBBatchTile = std::is_same<R, double>::value ? 2 : 3;
     static int batch_blocks_per_sm(int variant)
     {
         int n = 0;
@@ -318,7 +378,7 @@ struct OpsImpl {
     }
     static const Ops& table()
     {
-        static const Ops t{sizeof(S), Store<S>::kPlanes, sizeof(CuT<S>), &interior, &wall, &init, &read, &contact, &film, &batch_step,
+        static const Ops t{sizeof(S), Store<S>::kPlanes, sizeof(CuT<S>), &interior, &wall, &tile, &use_tile, &init, &read, &contact, &film, &batch_step,
                           &batch_blocks_per_sm, sizeof(LatDesc<R>), &fill_desc, &mass, &init_rows, sizeof(R),
                           &csum_ip, &interior_ip, &wall_ip, &swap_ip};
         return t;
