@@ -442,7 +442,12 @@ int tlb_set_params(tlb_lattice* L, const tlb_params* p)
         P.drho12[i] = P.drho[i] / 12.0;
         P.aM6[i] = P.aM[i] / 6.0;
         P.K3w3[i] = 3.0 * P.Kw3[i];
+        P.kqs[i] = P.kq[i] + P.ks[i];
+        P.Kl2[i] = 2.0 * P.Kl[i];
+        P.Kl3[i] = -3.0 * P.Kl[i];
     }
+    P.rho23 = -2.0 / 3.0 * p->rho3;
+    P.kp3 = 0.6 * P.p3tg3;
     P.Kt = P.k12D * P.two_lamT;
     // mu_1 - mu_3 = (1 + l3/l1) mu_1 + (l3/l2) mu_2, mu_2 - mu_3 = (l3/l1) mu_1 + (1 + l3/l2) mu_2
     P.qa[0][0] = (1.0 + P.l3_l1) / 12.0;

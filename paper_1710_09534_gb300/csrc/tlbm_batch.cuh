@@ -51,8 +51,13 @@ __device__ __noinline__ void batch_wall_item(const LatDesc<R>* d, int parity, co
                                              TileShared<R, TY>& sh)
 {
     const Geo g = d->g;
-    tile_step<S, R, TY, MRT, false, true>((const S*)d->buf[parity], (S*)d->buf[parity ^ 1], (CuT<S>*)d->cu, d->cls, g, P,
-                                          bx * 32, by * TY - tile_shift(g.edge[3] == EDGE_LID, g.ny, TY), sh);
+    const S* fA = (const S*)d->buf[parity];
+    S* fB = (S*)d->buf[parity ^ 1];
+    const int y0 = by * TY - tile_shift(g.edge[3] == EDGE_LID, g.ny, TY);
+    if (kLean<R> && P.uni != R(0))
+        tile_step<S, R, TY, MRT, kLean<R>, true>(fA, fB, (CuT<S>*)d->cu, d->cls, g, P, bx * 32, y0, sh);
+    else
+        tile_step<S, R, TY, MRT, false, true>(fA, fB, (CuT<S>*)d->cu, d->cls, g, P, bx * 32, y0, sh);
 }
 
 // The near-wall tiles go through the interior kernel's own queue, before the

@@ -313,7 +313,7 @@ __device__ __forceinline__ void interior_tile_ip(S* f, CuT<S>* __restrict__ cu, 
             if (!PREFETCH) load_all_f();
         }
         CollideOf<S, MRT, R, UNI> col;
-        col.build(P, m, h, c1ux - cp[0], c1uy - cp[1], c2ux - cp[2], c2uy - cp[3]);
+        col.build(P, m, h, cp[0], cp[1], cp[2], cp[3]);
         collide_all_inplace<S, R>(col, gv,
             [&](auto kc, R& f1k, R& f2k) {
                 if constexpr (kPre) {
@@ -416,14 +416,13 @@ __device__ __forceinline__ void wall_node_ip(S* f, CuT<S>* __restrict__ cu, cons
         Hydro<R> h;
         hydro_from_g(P, m, gv, h);
         const R c1ux = m.c1 * h.ux, c1uy = m.c1 * h.uy, c2ux = m.c2 * h.ux, c2uy = m.c2 * h.uy;
-        const R d1x = c1ux - R(cu[0 * PL + o]), d1y = c1uy - R(cu[1 * PL + o]);
-        const R d2x = c2ux - R(cu[2 * PL + o]), d2y = c2uy - R(cu[3 * PL + o]);
+        const R o1x = R(cu[0 * PL + o]), o1y = R(cu[1 * PL + o]), o2x = R(cu[2 * PL + o]), o2y = R(cu[3 * PL + o]);
         cu[0 * PL + o] = CuT<S>(c1ux);
         cu[1 * PL + o] = CuT<S>(c1uy);
         cu[2 * PL + o] = CuT<S>(c2ux);
         cu[3 * PL + o] = CuT<S>(c2uy);
         CollideOf<S, MRT, R> col;
-        col.build(P, m, h, d1x, d1y, d2x, d2y);
+        col.build(P, m, h, o1x, o1y, o2x, o2y);
         collide_all_inplace<S, R>(col, gv,
             [&](auto kc, R& f1k, R& f2k) {
                 constexpr int K = decltype(kc)::value;
@@ -450,14 +449,13 @@ __device__ __forceinline__ void wall_node_ip(S* f, CuT<S>* __restrict__ cu, cons
         h.uy = R(0);
         h.usq = P.lid_u * P.lid_u;
         const R c1ux = m.c1 * h.ux, c2ux = m.c2 * h.ux;
-        const R d1x = c1ux - R(cu[0 * PL + o]), d1y = R(0) - R(cu[1 * PL + o]);
-        const R d2x = c2ux - R(cu[2 * PL + o]), d2y = R(0) - R(cu[3 * PL + o]);
+        const R o1x = R(cu[0 * PL + o]), o1y = R(cu[1 * PL + o]), o2x = R(cu[2 * PL + o]), o2y = R(cu[3 * PL + o]);
         cu[0 * PL + o] = CuT<S>(c1ux);
         cu[1 * PL + o] = CuT<S>(0);
         cu[2 * PL + o] = CuT<S>(c2ux);
         cu[3 * PL + o] = CuT<S>(0);
         CollideOf<S, MRT, R> col;
-        col.build(P, m, h, d1x, d1y, d2x, d2y);
+        col.build(P, m, h, o1x, o1y, o2x, o2y);
         // Eq. 51: f(x_u) = f^eq(x_u) + [f(x_f) - f^eq(x_f)], for f^1, f^2 and g
         R gu[9], f1u[9], f2u[9];
 #pragma unroll

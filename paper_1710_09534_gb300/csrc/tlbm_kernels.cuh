@@ -900,7 +900,7 @@ __device__ __forceinline__ void interior_tile(const S* __restrict__ fA, S* __res
         cu[2 * PL + ou] = CuT<S>(c2ux);
         cu[3 * PL + ou] = CuT<S>(c2uy);
         CollideOf<S, MRT, R, UNI> col;
-        col.template build<SE>(P, m, h, c1ux - cp[0], c1uy - cp[1], c2ux - cp[2], c2uy - cp[3]);
+        col.template build<SE>(P, m, h, cp[0], cp[1], cp[2], cp[3]);
         const PushOffsets po(g, xs, yu);
         const int su = (yu + 9) % 3;
         collide_all<S, R, SE>(col, gv,

@@ -68,10 +68,15 @@ inline Prm<R> cast_prm(const Prm<double>& d)
         r.kq[i] = R(d.kq[i]);
         r.ks[i] = R(d.ks[i]);
         r.K3w3[i] = R(d.K3w3[i]);
+        r.kqs[i] = R(d.kqs[i]);
+        r.Kl2[i] = R(d.Kl2[i]);
+        r.Kl3[i] = R(d.Kl3[i]);
         r.qa[i][0] = R(d.qa[i][0]);
         r.qa[i][1] = R(d.qa[i][1]);
     }
     r.Kt = R(d.Kt);
+    r.rho23 = R(d.rho23);
+    r.kp3 = R(d.kp3);
     return r;
 }
 
@@ -155,9 +160,10 @@ struct OpsImpl {
                             int ntiles, const Geo& g, const Prm<double>& Pd, cudaStream_t s)
     {
         const Prm<R> P = cast_prm<R>(Pd);
+        auto* k = kLean<R> && Pd.uni != 0.0 ? &k_step_wall<S, R, MRT, kLean<R>> : &k_step_wall<S, R, MRT, false>;
         if (ntiles > 0)
-            k_step_wall<S, R, MRT><<<ntiles, 32 * kWallTY, 0, s>>>((const S*)fA, (S*)fB, (CuT<S>*)cu, cls, tiles, g, P,
-                                                                   tile_shift(g.edge[3] == EDGE_LID, g.ny, kWallTY));
+            k<<<ntiles, 32 * kWallTY, 0, s>>>((const S*)fA, (S*)fB, (CuT<S>*)cu, cls, tiles, g, P,
+                                              tile_shift(g.edge[3] == EDGE_LID, g.ny, kWallTY));
         return cudaGetLastError();
     }
     // A launch whose blocks may become resident while the launch before it in

@@ -23,7 +23,9 @@
 // The arithmetic of every node is that of the other two kernels, operation by
 // operation: interior nodes use the column sums (ColRings), the others the
 // window form with the ghost rules of Eqs. 42-43 (window_macros), whose mu is
-// kept apart (wm) because it rounds differently from the column form.
+// kept apart (wm) because it rounds differently from the column form.  Near-wall
+// nodes of a lattice of uniform properties take the general update in FP32
+// arithmetic and the uniform one in FP64.
 #pragma once
 #include "tlbm_kernels.cuh"
 
@@ -51,7 +53,7 @@ __device__ __forceinline__ auto tile_c(const TileShared<R, TY>& sh, int i, int j
 
 // Macros of the near-wall or lid-adjacent node at shared position (i, j):
 // window_macros with the window in shared memory.
-template <typename R, int TY>
+template <bool UNI, typename R, int TY>
 __device__ __forceinline__ void tile_macros(const TileShared<R, TY>& sh, const Prm<R>& P, int i, int j, Macro<R>& m)
 {
     R v1[9], v2[9], w1[9], w2[9];
@@ -78,9 +80,14 @@ __device__ __forceinline__ void tile_macros(const TileShared<R, TY>& sh, const P
     m.mu2 = w2[0];
     grad9s(v1, m.g1x, m.g1y);
     grad9s(v2, m.g2x, m.g2y);
-    m.lm1 = lap9s(w1);
-    m.lm2 = lap9s(w2);
-    m.rho = density(P, m.c1, m.c2);
+    if constexpr (UNI) {
+        m.lm1 = m.lm2 = R(0);
+        m.rho = P.rho[2];
+    } else {
+        m.lm1 = lap9s(w1);
+        m.lm2 = lap9s(w2);
+        m.rho = density(P, m.c1, m.c2);
+    }
 }
 
 // Class byte of site (x, y) (on an inside site with its wrapped offset), or
@@ -263,9 +270,11 @@ __device__ __forceinline__ void tile_step(const S* __restrict__ fA, S* __restric
     const int kind = mine & CLS_KIND_MASK;
     const PushOffsets po(g, x, y);
 
-    // Interior nodes with an update of their own (the uniform-property form, and
-    // the units of 16-bit storage): near-wall nodes take the general one below.
-    constexpr bool kSplit = UNI || SE != 0 || WALL;
+    // Interior nodes with an update of their own (FP32 arithmetic: the uniform-
+    // property form, and the units of 16-bit storage): near-wall nodes take the
+    // general one below.
+    constexpr bool kSplit = (UNI && !kLean<R>) || SE != 0 || WALL;
+    constexpr bool kUniWall = UNI && kLean<R>;
     const bool inner = (mine & CLS_INTERIOR) != 0;
     if (WALL && inner) return;
     Macro<R> m;
@@ -301,7 +310,7 @@ __device__ __forceinline__ void tile_step(const S* __restrict__ fA, S* __restric
             cu[2 * PL + o] = CuT<S>(c2ux);
             cu[3 * PL + o] = CuT<S>(c2uy);
             CollideOf<S, MRT, R, UNI> col;
-            col.template build<SE>(P, m, h, c1ux - cp[0], c1uy - cp[1], c2ux - cp[2], c2uy - cp[3]);
+            col.template build<SE>(P, m, h, cp[0], cp[1], cp[2], cp[3]);
             collide_all<S, R, SE>(col, gv,
                 [&](auto kc, R& f1k, R& f2k) {
                     f1k = f[decltype(kc)::value];
@@ -328,7 +337,7 @@ __device__ __forceinline__ void tile_step(const S* __restrict__ fA, S* __restric
     // where the update is the same, interior ones: a warp that holds both kinds
     // runs it once.  A lid node takes the macros of the row below it.
     const bool lid = kind == ST_LID;
-    if (kSplit || !inner) tile_macros(sh, P, tx + 2, ty + 2 - lid, m);
+    if (kSplit || !inner) tile_macros<kUniWall>(sh, P, tx + 2, ty + 2 - lid, m);
     const long long of = lid ? o - g.pitch : o;
     if (lid) {
 #pragma unroll
@@ -343,7 +352,7 @@ __device__ __forceinline__ void tile_step(const S* __restrict__ fA, S* __restric
         }
     }
     Hydro<R> h;
-    hydro_from_g(P, m, gv, h);
+    hydro_from_g<kUniWall>(P, m, gv, h);
     if (lid) {
         // Eq. 51: f(x_u) = f^eq(x_u) + [f(x_f) - f^eq(x_f)], for f^1, f^2 and g
         const R fx = h.ux, fy = h.uy;
@@ -373,8 +382,8 @@ __device__ __forceinline__ void tile_step(const S* __restrict__ fA, S* __restric
     cu[1 * PL + o] = CuT<S>(c1uy);
     cu[2 * PL + o] = CuT<S>(c2ux);
     cu[3 * PL + o] = CuT<S>(c2uy);
-    CollideOf<S, MRT, R> col;
-    col.build(P, m, h, c1ux - cp[0], c1uy - cp[1], c2ux - cp[2], c2uy - cp[3]);
+    CollideOf<S, MRT, R, kUniWall> col;
+    col.build(P, m, h, cp[0], cp[1], cp[2], cp[3]);
     collide_all<S, R>(col, gv,
         [&](auto kc, R& f1k, R& f2k) {
             f1k = f[decltype(kc)::value];
@@ -422,15 +431,15 @@ k_step_tile(const S* __restrict__ fA, S* __restrict__ fB, CuT<S>* __restrict__ c
 // from row -yshift on (tile_shift).  Short tiles, because the near-wall nodes of a straight
 // wall are two rows.
 // ---------------------------------------------------------------------------
-template <typename S, typename R, bool MRT>
+template <typename S, typename R, bool MRT, bool UNI>
 __global__ void __launch_bounds__(32 * kWallTY, 2)
 k_step_wall(const S* __restrict__ fA, S* __restrict__ fB, CuT<S>* __restrict__ cu, const uint8_t* __restrict__ cls,
             const uint32_t* __restrict__ tiles, Geo g, Prm<R> P, int yshift)
 {
     __shared__ TileShared<R, kWallTY> sh;
     const uint32_t w = tiles[blockIdx.x];
-    tile_step<S, R, kWallTY, MRT, false, true>(fA, fB, cu, cls, g, P, (int)(w & 0xffffu) * 32,
-                                               (int)(w >> 16) * kWallTY - yshift, sh);
+    tile_step<S, R, kWallTY, MRT, UNI, true>(fA, fB, cu, cls, g, P, (int)(w & 0xffffu) * 32,
+                                             (int)(w >> 16) * kWallTY - yshift, sh);
 }
 
 }  // namespace tlb
