@@ -1400,6 +1400,9 @@ int tlb3_read_fields(tlb3_lattice* L, uint32_t mask, double* host_out)
     const size_t N = (size_t)L->n();
     double* stage = L->stage();
     if ((rc = L->prec == TLB_FP32 ? read3_t<float>(L, stage) : read3_t<double>(L, stage))) return rc;
+    int planes = 0;
+    for (int q = 0; q < 11; q++) planes += (mask >> q) & 1u;
+    tlb::touch_host(host_out, (size_t)planes * N * sizeof(double));
     size_t done = 0;
     for (int q = 0; q < 11; q++) {
         if (!(mask & (1u << q))) continue;

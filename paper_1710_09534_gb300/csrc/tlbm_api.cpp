@@ -673,6 +673,9 @@ int tlb_read_fields(tlb_lattice* L, uint32_t mask, double* host_out)
                                         : (size_t)(L->ops->ndist * L->lay.plane * L->ops->elem);
     const int per_pass = (int)std::min<size_t>(10, spare / (N * 8));
     double* stage = (double*)(L->lay.inplace ? L->cpl() : L->bufB());
+    size_t planes = 0;
+    for (int q = 0; q < 10; q++) planes += (mask >> q) & 1u;
+    tlb::touch_host(host_out, planes * N * 8);
     size_t done = 0;
     for (int q = 0; q < 10;) {
         uint32_t sub = 0;

@@ -86,6 +86,16 @@ void batch_member_changed(tlb_batch* B);
 // batch steps still queued on it); TLB_OK for a lattice outside any batch.
 int batch_sync(tlb_batch* B);
 
+// Writes one byte of every page of a host buffer that is about to be filled by
+// copies from the device: the device takes the page faults of a fresh buffer
+// one by one (GB300, 170 MB of FP64 planes: 53 ms, after 5 ms of touching 1 ms).
+inline void touch_host(void* p, size_t bytes)
+{
+    volatile char* c = (volatile char*)p;
+    for (size_t i = 0; i < bytes; i += 4096) c[i] = 0;
+    if (bytes) c[bytes - 1] = 0;
+}
+
 // Record an error message for tlb_last_error() and return `code`.
 int set_error(int code, const char* msg);
 int clear_error();
