@@ -58,8 +58,8 @@ def storage_bytes_per_node(precision):
     return 2 * (25 * 2 + 4 * 4 + 4 * 4)
 
 
-KERNEL = {"fp64": "k_step_interior<double>", "fp32": "k_step_interior<float>",
-          "fp16": "k_step_interior<__half>", "bf16": "k_step_interior<__nv_bfloat16>"}
+KERNEL = {"fp64": "k_step_march<double>", "fp32": "k_step_interior<float>",
+          "fp16": "k_step_march<__half>", "bf16": "k_step_interior<__nv_bfloat16>"}
 
 
 # FP64 arithmetic per node update of the fused interior kernel as counted by
@@ -411,7 +411,7 @@ def run_ours(args):
                 "peak_source": peak_src,
                 "peak_nominal": round(FP64_PEAK_TFLOPS, 4),
                 "peak_nominal_source": "152 SMs x 2 DP inst/clk x 2 flop x 2.07 GHz",
-                "kernel": "k_step_interior<double>", "update": path,
+                "kernel": "k_step_march<double>", "update": path,
                 "dp_inst_per_node": dp_inst, "flops_per_node": dp_flops,
                 "dp_issue_frac": round(dp_issue, 4),
                 "hbm_achieved_gbs": round(ach_gbs, 1), "hbm_peak_gbs": hbm_gbs, "hbm_frac": round(hbm_frac, 4)}

@@ -192,15 +192,15 @@ int tlb_set_fields(tlb_lattice *lat, const double *c1, const double *c2, const d
 int tlb_set_fields_device(tlb_lattice *lat, const double *c1, const double *c2,
                           const double *ux, const double *uy, const double *p);
 
-/* Advance n >= 0 time steps, asynchronously on the stream: per step one fused
- * interior kernel and one near-wall kernel, or one kernel over all nodes where
- * that is faster (two-buffer lattices up to about 3.0, 1.4 and 0.75 million
- * nodes in FP64, FP32 and 16-bit storage); in-place lattices: the
+/* Advance n >= 0 time steps, asynchronously on the stream: one launch per
+ * step, over tiles up to about 3.0, 1.4 and 0.75 million nodes in FP64, FP32
+ * and 16-bit storage and in marching strips beyond; in-place lattices: the
  * order-parameter pass, the interior kernel, the lid row if any, the
  * near-wall kernel, and after a last even step the in-place streaming.  The
- * near-wall launches run on a stream the lattice owns, ordered after the
- * step's earlier work and joined back into the caller's stream before the
- * step ends, so work the caller queues after tlb_step sees the whole step.
+ * near-wall launches of an in-place lattice run on a stream the lattice owns,
+ * ordered after the step's earlier work and joined back into the caller's
+ * stream before the step ends, so work the caller queues after tlb_step sees
+ * the whole step.
  * TLB_ESTATE before set_fields. */
 int tlb_step(tlb_lattice *lat, int64_t n);
 
@@ -270,9 +270,9 @@ int tlb_theta12_from(double sigma12, double sigma13, double sigma23, double thet
  * starts recording events around the fused interior launch and the
  * near-wall launch of every step (and clears the totals); enable = 0 stops.
  * tlb_profile_read synchronizes and returns the summed device milliseconds
- * ms[0] (interior kernel), ms[1] (near-wall kernel) and the launch counts; a
- * lattice stepped by one kernel over all nodes reports it as the interior one,
- * with no near-wall launch. */
+ * ms[0] (interior kernel), ms[1] (near-wall kernel) and the launch counts;
+ * two-buffer lattices step by one launch, reported as the interior one, and
+ * have no near-wall launch. */
 int tlb_profile(tlb_lattice *lat, int enable);
 int tlb_profile_read(tlb_lattice *lat, double ms[2], int64_t launches[2]);
 

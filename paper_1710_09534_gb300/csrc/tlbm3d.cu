@@ -232,6 +232,7 @@ template <typename R>
 __global__ void k3_csum(const R* __restrict__ f, R* __restrict__ cpl, const uint8_t* __restrict__ kind,
                         Geo3 g)
 {
+    tlb::after_previous_launch();
     NODE_OF_THREAD
     const long long PL = g.plane;
     R a = R(0.0), b = R(0.0);
@@ -281,6 +282,7 @@ template <typename R>
 __global__ void k3_mu(const R* __restrict__ cpl, R* __restrict__ mpl, const uint32_t* __restrict__ lnk,
                       Geo3 g, Prm3<R> P)
 {
+    tlb::after_previous_launch();
     NODE_OF_THREAD
     const long long PL = g.plane;
     const uint32_t L = lnk[o];
@@ -718,6 +720,7 @@ k3_update(const R* __restrict__ fA, R* __restrict__ fB, R* __restrict__ cu,
           const R* __restrict__ cpl, const R* __restrict__ mpl, const uint32_t* __restrict__ lnk, Geo3 g,
           Prm3<R> P)
 {
+    tlb::after_previous_launch();
     NODE_OF_THREAD
     const long long PL = g.plane;
     if constexpr (kStage3<R>) {
@@ -1053,12 +1056,13 @@ int prof_mark3(tlb3_lattice* L, int j)
 template <typename R>
 int order_params3_t(tlb3_lattice* L, bool in_step)
 {
-    tlb3::k3_csum<R><<<grid3(L), 128, 0, L->stream>>>(L->fcur<R>(), L->cpl<R>(), L->kind(), L->geo);
+    T3_CUDA(tlb::launch_dependent(&tlb3::k3_csum<R>, grid3(L), 128, 0, L->stream, (const R*)L->fcur<R>(), L->cpl<R>(),
+                                  (const uint8_t*)L->kind(), L->geo));
     int rc = prof_mark3(L, 1);
     if (rc) return rc;
     if (!(in_step && L->uni && tlb3::kFuseMu3<R>))
-        tlb3::k3_mu<R><<<grid3(L), 128, 0, L->stream>>>(L->cpl<R>(), L->mpl<R>(), L->lnk(), L->geo, L->P<R>());
-    T3_CUDA(cudaGetLastError());
+        T3_CUDA(tlb::launch_dependent(&tlb3::k3_mu<R>, grid3(L), 128, 0, L->stream, (const R*)L->cpl<R>(), L->mpl<R>(),
+                                      (const uint32_t*)L->lnk(), L->geo, L->P<R>()));
     return TLB_OK;
 }
 int order_params3(tlb3_lattice* L, bool in_step = false)
@@ -1078,15 +1082,10 @@ int update3_t(tlb3_lattice* L)
         T3_CUDA(cudaFuncSetAttribute(tlb3::k3_update<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
         L->stage_attr = true;
     }
-    if (L->uni)
-        tlb3::k3_update<R, true><<<grid3(L), 128, dyn, L->stream>>>(L->fcur<R>(), L->fspare<R>(), L->cu<R>(),
-                                                                    L->cpl<R>(), L->mpl<R>(), L->lnk(), L->geo,
-                                                                    L->P<R>());
-    else
-        tlb3::k3_update<R, false><<<grid3(L), 128, dyn, L->stream>>>(L->fcur<R>(), L->fspare<R>(), L->cu<R>(),
-                                                                     L->cpl<R>(), L->mpl<R>(), L->lnk(), L->geo,
-                                                                     L->P<R>());
-    T3_CUDA(cudaGetLastError());
+    auto* k = L->uni ? &tlb3::k3_update<R, true> : &tlb3::k3_update<R, false>;
+    T3_CUDA(tlb::launch_dependent(k, grid3(L), 128, dyn, L->stream, (const R*)L->fcur<R>(), L->fspare<R>(), L->cu<R>(),
+                                  (const R*)L->cpl<R>(), (const R*)L->mpl<R>(), (const uint32_t*)L->lnk(), L->geo,
+                                  L->P<R>()));
     return TLB_OK;
 }
 

@@ -162,9 +162,6 @@ int build_geometry(tlb_lattice* L)
     return TLB_OK;
 }
 
-// Whether a step of this lattice is one launch over all its nodes.
-bool one_launch(const tlb_lattice* L) { return !L->lay.inplace && L->ops->use_tile(L->n()); }
-
 constexpr int kProfSlots = 512;
 
 // Fold the recorded events (per step: interior start/end, near-wall
@@ -181,7 +178,7 @@ int prof_fold(tlb_lattice* L)
         L->prof_ms[0] += a;
         L->prof_ms[1] += b;
         L->prof_n[0] += 1;
-        L->prof_n[1] += L->nlist > 0 && !one_launch(L) ? 1 : 0;
+        L->prof_n[1] += L->lay.inplace && L->nlist > 0 ? 1 : 0;
     }
     L->ev_used = 0;
     return TLB_OK;
@@ -605,26 +602,16 @@ int tlb_step(tlb_lattice* L, int64_t n)
     if (!L->have_params || !L->have_fields) return fail(TLB_ESTATE, "set_params and set_fields before step");
     if (L->batch) return fail(TLB_ESTATE, "lattice belongs to a batch: step the batch");
     if (L->lay.inplace) return step_inplace(L, n);
-    if (one_launch(L)) {
-        for (int64_t s = 0; s < n; s++) {
-            rc = step_launches(
-                L, false, [] { return cudaSuccess; },
-                [&] { return L->ops->tile(L->bufA(), L->bufB(), L->cu(), L->dcls(), L->geo, L->prm, L->stream); },
-                [](cudaStream_t) { return cudaSuccess; }, [] { return cudaSuccess; });
-            if (rc) return rc;
-            L->cur ^= 1;
-        }
-        return ok();
-    }
+    const bool tile = L->ops->use_tile(L->n());
     for (int64_t s = 0; s < n; s++) {
         rc = step_launches(
-            L, L->nlist > 0, [] { return cudaSuccess; },
-            [&] { return L->ops->interior(L->bufA(), L->bufB(), L->cu(), L->dcls(), L->geo, L->prm, L->stream); },
-            [&](cudaStream_t ws) {
-                return L->ops->wall(L->bufA(), L->bufB(), L->cu(), L->dcls(), L->dlist(), (int)L->nwork, L->geo,
-                                    L->prm, ws);
+            L, false, [] { return cudaSuccess; },
+            [&] {
+                return tile ? L->ops->tile(L->bufA(), L->bufB(), L->cu(), L->dcls(), L->geo, L->prm, L->stream)
+                            : L->ops->march(L->bufA(), L->bufB(), L->cu(), L->dcls(), L->dlist(), (int)L->nwork, L->geo,
+                                            L->prm, L->stream);
             },
-            [] { return cudaSuccess; });
+            [](cudaStream_t) { return cudaSuccess; }, [] { return cudaSuccess; });
         if (rc) return rc;
         L->cur ^= 1;
     }

@@ -5,7 +5,7 @@
 // launch:
 //   k_batch_interior: a persistent kernel whose blocks take items from a shared
 //                     counter until the list is exhausted: first the members'
-//                     near-wall tiles (k_step_wall's code), then their interior
+//                     near-wall tiles (wall_tile), then their interior
 //                     tiles (member, strip, segment), running the same tile
 //                     code as the single-lattice kernels;
 //   k_batch_tile:     for batches whose members together are small enough for
@@ -44,22 +44,6 @@ struct BatchCounters {
     int next, done;  // items taken and blocks finished of the running launch (zero between launches)
 };
 
-// One near-wall tile of a member; a call of its own, so that its registers are
-// not the interior update's (inlined, FP64 spilled 40 words and FP16 100).
-template <typename S, typename R, int TY, bool MRT>
-__device__ __noinline__ void batch_wall_item(const LatDesc<R>* d, int parity, const Prm<R>& P, int bx, int by,
-                                             TileShared<R, TY>& sh)
-{
-    const Geo g = d->g;
-    const S* fA = (const S*)d->buf[parity];
-    S* fB = (S*)d->buf[parity ^ 1];
-    const int y0 = by * TY - tile_shift(g.edge[3] == EDGE_LID, g.ny, TY);
-    if (kLean<R> && P.uni != R(0))
-        tile_step<S, R, TY, MRT, kLean<R>, true>(fA, fB, (CuT<S>*)d->cu, d->cls, g, P, bx * 32, y0, sh);
-    else
-        tile_step<S, R, TY, MRT, false, true>(fA, fB, (CuT<S>*)d->cu, d->cls, g, P, bx * 32, y0, sh);
-}
-
 // The near-wall tiles go through the interior kernel's own queue, before the
 // interior tiles: as a launch of their own beside it they either waited for
 // the persistent blocks, which fill every register file, or kept some of them
@@ -72,22 +56,14 @@ k_batch_interior(const LatDesc<R>* __restrict__ descs, const TileItem* __restric
 {
     constexpr int WTY = BLOCK / 32;
     constexpr bool kStash = kStashPops && std::is_same<R, float>::value && !kDenseMrt<S, MRT>;
-    struct March {
-        ColRings<R, BLOCK> rings;
-        PopStash<R, kStash ? BLOCK : 1> stash;
-    };
-    // an item is either kind, so its shared data share one place
-    constexpr size_t kBytes = sizeof(March) > sizeof(TileShared<R, WTY>) ? sizeof(March) : sizeof(TileShared<R, WTY>);
-    __shared__ __align__(16) unsigned char raw[kBytes];
-    March& sh = *reinterpret_cast<March*>(raw);
+    __shared__ MarchShared<R, BLOCK, kStash> sh;
     __shared__ Prm<R> Ps;
     __shared__ int item_s;
     static_assert(sizeof(Prm<R>) % sizeof(R) == 0, "params are whole words");
     constexpr int kWords = (int)(sizeof(Prm<R>) / sizeof(R));
     const int nw = ctr->n_wall, n = nw + ctr->n_tiles;
     // the state, and the counters, are those of the previous launch
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    after_previous_launch();
     for (;;) {
         if (threadIdx.x == 0) item_s = atomicAdd(&ctr->next, 1);
         __syncthreads();
@@ -106,15 +82,15 @@ k_batch_interior(const LatDesc<R>* __restrict__ descs, const TileItem* __restric
         CuT<S>* cu = (CuT<S>*)d->cu;
         // members with equal densities and viscosities take the uniform-property
         // update, as they do when stepped alone (the branch is uniform per tile)
-        auto* st = reinterpret_cast<PopStash<R, BLOCK>*>(&sh.stash);  // used only when kStash
+        auto* st = reinterpret_cast<PopStash<R, BLOCK>*>(&sh.m.stash);  // used only when kStash
         if (wall)
-            batch_wall_item<S, R, WTY, MRT>(d, parity, Ps, ti.bx, ti.by, *reinterpret_cast<TileShared<R, WTY>*>(raw));
+            wall_tile<S, R, WTY, MRT>(fA, fB, cu, d->cls, g, Ps, ti.bx, ti.by, sh.tile);
         else if (Ps.uni != R(0))
             interior_tile<S, R, BLOCK, PREFETCH, MRT, true, kStash>(fA, fB, cu, d->cls, g, Ps, ti.bx, ti.by, d->rows,
-                                                                    sh.rings, st);
+                                                                    sh.m.rings, st);
         else
             interior_tile<S, R, BLOCK, PREFETCH, MRT, false, kStash>(fA, fB, cu, d->cls, g, Ps, ti.bx, ti.by, d->rows,
-                                                                     sh.rings, st);
+                                                                     sh.m.rings, st);
         __syncthreads();  // shared data, parameters and item_s are reused by the next item
     }
     // the last block leaves the counters as the next launch expects them

@@ -39,7 +39,7 @@ struct Geo {
     long long plane;  // elements per plane = ny * pitch
 };
 
-// Rows of a near-wall tile (k_step_wall), and the rows by which the first tile
+// Rows of a near-wall tile (k_step_march), and the rows by which the first tile
 // of height ty starts below row 0, so that a lid row never is the first row of
 // its tile (its window reaches three rows down).
 constexpr int kWallTY = 4;
@@ -735,7 +735,29 @@ struct MrtNode {
     }
 };
 
-template <typename S>
-__device__ __forceinline__ S ldg(const S* p) { return __ldg(p); }
+// Programmatic dependent launch: launch_dependent's blocks may become resident
+// while the launch before them in the stream finishes; after_previous_launch
+// waits until that one is complete and lets the next one start its blocks.
+// What a kernel reads before it must not be written by an earlier step.
+__device__ __forceinline__ void after_previous_launch()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <typename K, typename... A>
+inline cudaError_t launch_dependent(K k, dim3 grid, int threads, size_t shared, cudaStream_t s, A... args)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = shared;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, args...);
+}
 
 }  // namespace tlb

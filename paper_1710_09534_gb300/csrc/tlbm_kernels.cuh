@@ -1,7 +1,7 @@
 // Kernels of one time step and of set-up / read-out, templated on the storage
 // type S and the arithmetic type R (double/double or float/float).
 //
-//   k_step_interior  fused stencil + collide + push for every node whose
+//   interior_tile    fused stencil + collide + push for every node whose
 //                    5x5 neighbourhood is plain fluid (no wall, no lid):
 //                    c_1, c_2 on the tile plus a radius-2 halo from the local
 //                    sums of the pre-collision f (push streaming keeps them
@@ -938,21 +938,6 @@ __device__ __forceinline__ void interior_tile(const S* __restrict__ fA, S* __res
                 st_lo(fB, 0, PL, ou, l1);
                 st_lo(fB, 1, PL, ou, l2);
             });
-    }
-}
-
-template <typename S, typename R, int BLOCK, int ROWS, bool PREFETCH, int MINB, bool MRT, bool UNI>
-__global__ void __launch_bounds__(BLOCK, MINB)
-k_step_interior(const S* __restrict__ fA, S* __restrict__ fB, CuT<S>* __restrict__ cu,
-                const uint8_t* __restrict__ cls, Geo g, Prm<R> P, int rows)
-{
-    __shared__ ColRings<R, BLOCK> sh;
-    if constexpr (kStashPops && std::is_same<R, float>::value && !kDenseMrt<S, MRT>) {
-        __shared__ PopStash<R, BLOCK> stash;
-        interior_tile<S, R, BLOCK, PREFETCH, MRT, UNI, true>(fA, fB, cu, cls, g, P, blockIdx.x, blockIdx.y, rows, sh,
-                                                            &stash);
-    } else {
-        interior_tile<S, R, BLOCK, PREFETCH, MRT, UNI>(fA, fB, cu, cls, g, P, blockIdx.x, blockIdx.y, rows, sh);
     }
 }
 

@@ -12,13 +12,11 @@ struct Ops {
     size_t elem;     // bytes per stored distribution scalar
     int ndist;       // planes of `elem` bytes per distribution buffer
     size_t cu_elem;  // bytes per scalar of the c_i u planes
-    // one time step A -> B = interior tiles (fused kernel) + near-wall list
-    cudaError_t (*interior)(const void* fA, void* fB, void* cu, const uint8_t* cls, const Geo& g,
-                            const Prm<double>& P, cudaStream_t s);
-    // (near-wall tiles, see k_step_wall)
-    cudaError_t (*wall)(const void* fA, void* fB, void* cu, const uint8_t* cls, const uint32_t* tiles,
-                        int ntiles, const Geo& g, const Prm<double>& P, cudaStream_t s);
-    // the same step in one launch (k_step_tile), for lattices (or batches) of few enough nodes (use_tile)
+    // one time step A -> B: the near-wall tiles `walls` and the interior tiles
+    // (k_step_march)
+    cudaError_t (*march)(const void* fA, void* fB, void* cu, const uint8_t* cls, const uint32_t* walls, int nwalls,
+                         const Geo& g, const Prm<double>& P, cudaStream_t s);
+    // the same step by tiles (k_step_tile), for lattices (or batches) of few enough nodes (use_tile)
     cudaError_t (*tile)(const void* fA, void* fB, void* cu, const uint8_t* cls, const Geo& g, const Prm<double>& P,
                         cudaStream_t s);
     bool (*use_tile)(long long nodes);
@@ -74,7 +72,7 @@ inline int ndist_for(int precision) { return precision == 0 ? 27 : (precision ==
 inline size_t cu_elem_for(int precision) { return precision == 0 ? 8 : 4; }
 
 // Tiles of 32 x ty nodes (row << 16 | column, in order) that hold any of the
-// near-wall nodes `list` (y << 16 | x); k_step_wall: ty = kWallTY.
+// near-wall nodes `list` (y << 16 | x); k_step_march: ty = kWallTY.
 std::vector<uint32_t> wall_tiles(const std::vector<uint32_t>& list, const Geo& g, int ty);
 
 const Ops& ops_f64();

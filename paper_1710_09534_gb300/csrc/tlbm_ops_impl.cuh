@@ -136,51 +136,20 @@ inline int rows_for(const Geo& g, int tx, int rows, int per_sm, bool one_wave = 
 template <typename S, typename R, int BLOCK, int ROWS, bool PREFETCH, int MINB, bool MRT>
 struct OpsImpl {
     static constexpr int kMinBUni = std::is_same<R, double>::value && !MRT ? TLB_MINB64_UNI : MINB;
-    static cudaError_t interior(const void* fA, void* fB, void* cu, const uint8_t* cls, const Geo& g,
-                                const Prm<double>& Pd, cudaStream_t s)
+    static cudaError_t march(const void* fA, void* fB, void* cu, const uint8_t* cls, const uint32_t* walls, int nwalls,
+                             const Geo& g, const Prm<double>& Pd, cudaStream_t s)
     {
         const Prm<R> P = cast_prm<R>(Pd);
         constexpr int TX = BLOCK - 4;
-        constexpr bool kOneWave = std::is_same<R, double>::value;
+        static_assert(BLOCK == 32 * kWallTY, "a block takes a strip segment or a near-wall tile");
         // equal densities and viscosities: the uniform-property update
-        if (Pd.uni != 0.0) {
-            const int rows = rows_for(g, TX, ROWS, kMinBUni, kOneWave);
-            dim3 grid((g.nx + TX - 1) / TX, (g.ny + rows - 1) / rows);
-            k_step_interior<S, R, BLOCK, ROWS, PREFETCH, kMinBUni, MRT, true><<<grid, BLOCK, 0, s>>>(
-                (const S*)fA, (S*)fB, (CuT<S>*)cu, cls, g, P, rows);
-        } else {
-            const int rows = rows_for(g, TX, ROWS, MINB, kOneWave);
-            dim3 grid((g.nx + TX - 1) / TX, (g.ny + rows - 1) / rows);
-            k_step_interior<S, R, BLOCK, ROWS, PREFETCH, MINB, MRT, false><<<grid, BLOCK, 0, s>>>(
-                (const S*)fA, (S*)fB, (CuT<S>*)cu, cls, g, P, rows);
-        }
-        return cudaGetLastError();
-    }
-    static cudaError_t wall(const void* fA, void* fB, void* cu, const uint8_t* cls, const uint32_t* tiles,
-                            int ntiles, const Geo& g, const Prm<double>& Pd, cudaStream_t s)
-    {
-        const Prm<R> P = cast_prm<R>(Pd);
-        auto* k = kLean<R> && Pd.uni != 0.0 ? &k_step_wall<S, R, MRT, kLean<R>> : &k_step_wall<S, R, MRT, false>;
-        if (ntiles > 0)
-            k<<<ntiles, 32 * kWallTY, 0, s>>>((const S*)fA, (S*)fB, (CuT<S>*)cu, cls, tiles, g, P,
-                                              tile_shift(g.edge[3] == EDGE_LID, g.ny, kWallTY));
-        return cudaGetLastError();
-    }
-    // A launch whose blocks may become resident while the launch before it in
-    // the stream finishes (the kernel waits for it: griddepcontrol.wait).
-    template <typename K, typename... A>
-    static cudaError_t launch_dependent(K k, dim3 grid, int threads, cudaStream_t s, A... args)
-    {
-        cudaLaunchAttribute at{};
-        at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        at.val.programmaticStreamSerializationAllowed = 1;
-        cudaLaunchConfig_t cfg{};
-        cfg.gridDim = grid;
-        cfg.blockDim = dim3(threads);
-        cfg.stream = s;
-        cfg.attrs = &at;
-        cfg.numAttrs = 1;
-        return cudaLaunchKernelEx(&cfg, k, args...);
+        const bool uni = Pd.uni != 0.0;
+        const int rows = rows_for(g, TX, ROWS, uni ? kMinBUni : MINB, std::is_same<R, double>::value);
+        const int strips = (g.nx + TX - 1) / TX, segs = (g.ny + rows - 1) / rows;
+        auto* k = uni ? &k_step_march<S, R, BLOCK, PREFETCH, kMinBUni, MRT, true>
+                      : &k_step_march<S, R, BLOCK, PREFETCH, MINB, MRT, false>;
+        return launch_dependent(k, dim3(nwalls + strips * segs), BLOCK, 0, s, (const S*)fA, (S*)fB, (CuT<S>*)cu, cls,
+                                walls, nwalls, strips, g, P, rows);
     }
     template <int TY, int MB>
     static cudaError_t launch_tile(const void* fA, void* fB, void* cu, const uint8_t* cls, const Geo& g,
@@ -190,7 +159,7 @@ struct OpsImpl {
         const int shift = tile_shift(g.edge[3] == EDGE_LID, g.ny, TY);
         const dim3 grid((g.nx + 31) / 32, (g.ny + shift + TY - 1) / TY);
         auto* k = Pd.uni != 0.0 ? &k_step_tile<S, R, TY, MB, MRT, true> : &k_step_tile<S, R, TY, MB, MRT, false>;
-        return launch_dependent(k, grid, 32 * TY, s, (const S*)fA, (S*)fB, (CuT<S>*)cu, cls, g, P, shift);
+        return launch_dependent(k, grid, 32 * TY, 0, s, (const S*)fA, (S*)fB, (CuT<S>*)cu, cls, g, P, shift);
     }
     // Tile height and resident blocks, GB300, us per step (4 x 2: TY = 4 at 2
     // blocks per SM, and so on):
@@ -273,10 +242,10 @@ struct OpsImpl {
         const WallItem* wi = (const WallItem*)walls;
         BatchCounters* c = (BatchCounters*)ctr;
         if (variant == 2)
-            return launch_dependent(&k_batch_tile<S, R, kMinBBatchTile, MRT>, dim3(grid), 32 * kBatchTY, s, d, ti, parity);
+            return launch_dependent(&k_batch_tile<S, R, kMinBBatchTile, MRT>, dim3(grid), 32 * kBatchTY, 0, s, d, ti, parity);
         if (variant == 0)
-            return launch_dependent(&k_batch_interior<S, R, 64, PREFETCH, kMinB64, MRT>, dim3(grid), 64, s, d, ti, wi, c, parity);
-        return launch_dependent(&k_batch_interior<S, R, 128, PREFETCH, MINB, MRT>, dim3(grid), 128, s, d, ti, wi, c, parity);
+            return launch_dependent(&k_batch_interior<S, R, 64, PREFETCH, kMinB64, MRT>, dim3(grid), 64, 0, s, d, ti, wi, c, parity);
+        return launch_dependent(&k_batch_interior<S, R, 128, PREFETCH, MINB, MRT>, dim3(grid), 128, 0, s, d, ti, wi, c, parity);
     }
     static constexpr int kMinBBatchTile = std::is_same<R, double>::value ? 2 : 3;
     static int batch_blocks_per_sm(int variant)
@@ -384,7 +353,7 @@ struct OpsImpl {
     }
     static const Ops& table()
     {
-        static const Ops t{sizeof(S), Store<S>::kPlanes, sizeof(CuT<S>), &interior, &wall, &tile, &use_tile, &init, &read, &contact, &film, &batch_step,
+        static const Ops t{sizeof(S), Store<S>::kPlanes, sizeof(CuT<S>), &march, &tile, &use_tile, &init, &read, &contact, &film, &batch_step,
                           &batch_blocks_per_sm, sizeof(LatDesc<R>), &fill_desc, &mass, &init_rows, sizeof(R),
                           &csum_ip, &interior_ip, &wall_ip, &swap_ip};
         return t;

@@ -1,6 +1,7 @@
 // One launch per time step for lattices that leave the marching kernel and
 // its near-wall companion bound by latency.
 //
+//   k_step_march  large lattices (below)
 //   k_step_tile  every node of a 32 x TY tile, one thread each, near-wall and
 //                lid nodes included: c_1, c_2 and the node classes of the tile
 //                plus two nodes around it go to shared memory once, the column
@@ -8,13 +9,13 @@
 //                from them, and every node then takes the update its class
 //                asks for.
 //
-// The marching kernel (k_step_interior) serialises the rows of a segment, and
-// a near-wall thread of k_step_wall sums the order parameters of its whole
-// 5x5 window by itself (450 loads and, in FP64, 25 times the additions; an
-// FP64 instruction of a warp takes 64 cycles of its scheduler on GB300,
-// however few lanes are active).  On a large lattice neither shows; on a
-// small one a step lasted as long as one segment and one such window.  Here
-// every c is summed once per tile, and the launches of successive steps overlap
+// The marching kernel serialises the rows of a segment, and a thread of the
+// former near-wall kernel summed the order parameters of its whole 5x5 window
+// by itself (450 loads and, in FP64, 25 times the additions; an FP64
+// instruction of a warp takes 64 cycles of its scheduler on GB300, however few
+// lanes are active).  On a large lattice neither shows; on a small one a step
+// lasted as long as one segment and one such window.  Here every c is summed
+// once per tile, and the launches of successive steps overlap
 // (programmatic dependent launch: a block classifies its sites while the
 // previous step finishes, then waits for it; 128x64 FP32 6.2 -> 3.7 us per
 // step).  GB300, us per step, the two kernels against this one: 128x64 FP64
@@ -147,10 +148,7 @@ __device__ __forceinline__ void tile_step(const S* __restrict__ fA, S* __restric
     const int mine = tile_site(g, cls, x, y, oo);
     // the state is that of the previous launch, which may still be running
     // (programmatic dependent launch); the next one may start its own prologue
-    if constexpr (!WALL) {
-        asm volatile("griddepcontrol.wait;" ::: "memory");
-        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    }
+    if constexpr (!WALL) after_previous_launch();
 
     // the thread's own node: everything its update reads, and its c
     R f[18], lo[2] = {R(0), R(0)}, gv[9], cp[4];
@@ -426,20 +424,58 @@ k_step_tile(const S* __restrict__ fA, S* __restrict__ fB, CuT<S>* __restrict__ c
 }
 
 // ---------------------------------------------------------------------------
-// K2: the near-wall and lid nodes beside k_step_interior, by tiles that hold
-// any: tiles[b] = (row of tiles << 16) | column of tiles, of 32 x kWallTY nodes
-// from row -yshift on (tile_shift).  Short tiles, because the near-wall nodes of a straight
-// wall are two rows.
+// One near-wall tile: column bx, row by of the tiles of 32 x TY nodes from row
+// -tile_shift on.  A call of its own, so that its registers are not those of
+// the interior update that shares its kernel (inlined into the batch kernel,
+// FP64 spilled 40 words and FP16 100).
 // ---------------------------------------------------------------------------
-template <typename S, typename R, bool MRT, bool UNI>
-__global__ void __launch_bounds__(32 * kWallTY, 2)
-k_step_wall(const S* __restrict__ fA, S* __restrict__ fB, CuT<S>* __restrict__ cu, const uint8_t* __restrict__ cls,
-            const uint32_t* __restrict__ tiles, Geo g, Prm<R> P, int yshift)
+template <typename S, typename R, int TY, bool MRT>
+__device__ __noinline__ void wall_tile(const S* fA, S* fB, CuT<S>* cu, const uint8_t* cls, const Geo& g, const Prm<R>& P,
+                                       int bx, int by, TileShared<R, TY>& sh)
 {
-    __shared__ TileShared<R, kWallTY> sh;
-    const uint32_t w = tiles[blockIdx.x];
-    tile_step<S, R, kWallTY, MRT, UNI, true>(fA, fB, cu, cls, g, P, (int)(w & 0xffffu) * 32,
-                                             (int)(w >> 16) * kWallTY - yshift, sh);
+    const int y0 = by * TY - tile_shift(g.edge[3] == EDGE_LID, g.ny, TY);
+    if (kLean<R> && P.uni != R(0))
+        tile_step<S, R, TY, MRT, kLean<R>, true>(fA, fB, cu, cls, g, P, bx * 32, y0, sh);
+    else
+        tile_step<S, R, TY, MRT, false, true>(fA, fB, cu, cls, g, P, bx * 32, y0, sh);
+}
+
+// Shared data of a block that takes either kind of work.
+template <typename R, int BLOCK, bool STASH>
+union __align__(16) MarchShared {
+    struct {
+        ColRings<R, BLOCK> rings;
+        PopStash<R, STASH ? BLOCK : 1> stash;
+    } m;
+    TileShared<R, BLOCK / 32> tile;
+    __device__ MarchShared() {}
+};
+
+// One step of a large lattice: block b < nwalls takes near-wall tile walls[b]
+// ((row << 16) | column, tiles of 32 x kWallTY nodes: short, because the
+// near-wall nodes of a straight wall are two rows), the others a strip segment
+// of the interior (interior_tile).  One launch, which overlaps the end of the
+// step before it; as two launches on two streams between events, GB300, us per
+// step: 2048^2 FP32 209.0 -> 204.7, FP16 149.8 -> 147.0, 1024x2048
+// impact FP32 113.1 -> 111.9.
+template <typename S, typename R, int BLOCK, bool PREFETCH, int MINB, bool MRT, bool UNI>
+__global__ void __launch_bounds__(BLOCK, MINB)
+k_step_march(const S* __restrict__ fA, S* __restrict__ fB, CuT<S>* __restrict__ cu, const uint8_t* __restrict__ cls,
+             const uint32_t* __restrict__ walls, int nwalls, int strips, const __grid_constant__ Geo g,
+             const __grid_constant__ Prm<R> P, int rows)
+{
+    constexpr bool kStash = kStashPops && std::is_same<R, float>::value && !kDenseMrt<S, MRT>;
+    __shared__ MarchShared<R, BLOCK, kStash> sh;
+    after_previous_launch();
+    const int b = (int)blockIdx.x - nwalls;
+    if (b < 0) {
+        const uint32_t w = walls[blockIdx.x];
+        wall_tile<S, R, BLOCK / 32, MRT>(fA, fB, cu, cls, g, P, (int)(w & 0xffffu), (int)(w >> 16), sh.tile);
+        return;
+    }
+    auto* st = reinterpret_cast<PopStash<R, BLOCK>*>(&sh.m.stash);  // used only when kStash
+    interior_tile<S, R, BLOCK, PREFETCH, MRT, UNI, kStash>(fA, fB, cu, cls, g, P, b % strips, b / strips, rows,
+                                                           sh.m.rings, st);
 }
 
 }  // namespace tlb

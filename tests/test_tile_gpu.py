@@ -1,9 +1,8 @@
 """The one-launch step of small lattices (k_step_tile) at the edges of its tiles.
 
 Stepped alone, lattices of these sizes take k_step_tile.  As members of a batch
-that also holds a large lattice they take the marching interior kernel and its
-near-wall items, and the large lattice stepped alone takes the marching kernel
-and k_step_wall.  All run the same arithmetic, so the raw states must be equal
+that also holds a large lattice they take the marching items and near-wall tiles
+of k_batch_interior, and the large lattice stepped alone takes k_step_march.  All run the same arithmetic, so the raw states must be equal
 bit for bit, for every storage, collision model, edge kind and ragged size; so
 must those of a batch of small lattices only (k_batch_tile).  In FP64 the state
 also equals the oracle within the parity bound.
