@@ -339,15 +339,17 @@ constexpr bool kGReg3 = !kLo3<R>;
 // from: global memory (plane stride PL, element o), or, with STG, the
 // block's shared-memory stage (stride = block size, element = thread) that
 // the update fills by asynchronous copies at its start; ready() waits for
-// this thread's copies.
-template <typename R, bool STG>
+// this thread's copies (STG 1) or for those of the whole block (STG 2; every
+// thread of the block calls it once, wherever it then is).
+template <typename R, int STG>
 struct PopSrc {
     const R* b;  // plane 0 of the node
     long long pl;
     __device__ __forceinline__ R operator()(int q) const { return b[q * pl]; }
     __device__ __forceinline__ void ready() const
     {
-        if constexpr (STG) asm volatile("cp.async.wait_all;" ::: "memory");
+        if constexpr (STG != 0) asm volatile("cp.async.wait_all;" ::: "memory");
+        if constexpr (STG == 2) asm volatile("barrier.sync 0;" ::: "memory");
     }
 };
 
@@ -361,7 +363,7 @@ struct Node3 {
     R g[Q];
 };
 
-template <bool UNI, typename R, bool STG, bool FUSE_MU = false>
+template <bool UNI, typename R, int STG, bool FUSE_MU = false>
 __device__ __forceinline__ void node3(const Geo3& g, const Prm3<R>& P, const PopSrc<R, STG>& fs,
                                       const R* __restrict__ cpl, const R* __restrict__ mpl, uint32_t L,
                                       const Nb3& nb, long long o, Node3<R>& n)
@@ -482,7 +484,7 @@ struct Coll3 {
     R wa36;
 };
 
-template <bool UNI, int p, typename R, bool STG>
+template <bool UNI, int p, typename R, int STG>
 __device__ __forceinline__ void pair3(const Coll3<R>& C, const PopSrc<R, STG>& fs, R* __restrict__ fB,
                                       const Node3<R>& n, const Nb3& nb, uint32_t L, long long o, long long PL,
                                       R& d1, R& d2)
@@ -603,7 +605,7 @@ __device__ __forceinline__ void cp_async(unsigned dst, const void* src)
     asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(dst), "l"(src), "n"(N) : "memory");
 }
 
-template <typename R, bool UNI, bool STG>
+template <typename R, bool UNI, int STG>
 __device__ __forceinline__ void update3_node(const PopSrc<R, STG>& fs, const PopSrc<R, STG>& cs, R* __restrict__ fB,
                                              R* __restrict__ cu, const R* __restrict__ cpl,
                                              const R* __restrict__ mpl, uint32_t L, const Geo3& g, int x, int y,
@@ -741,7 +743,7 @@ k3_update(const R* __restrict__ fA, R* __restrict__ fB, R* __restrict__ cu,
         for (int q = 0; q < kPlanes3<R>; q++) cp_async<E>(sb + E * 128u * q, fA + q * PL + o);
 #pragma unroll
         for (int a = 0; a < 6; a++) cp_async<E>(sb + E * 128u * (kPlanes3<R> + a), cu + a * PL + o);
-        const PopSrc<R, true> fs{&stg[0][t], 128}, cs{&stg[kPlanes3<R>][t], 128};
+        const PopSrc<R, 1> fs{&stg[0][t], 128}, cs{&stg[kPlanes3<R>][t], 128};
         const uint32_t L = lnk[o];
         if (L & LNK_SOLID) {
             fs.ready();  // no copy into the stage may outlive the block
@@ -751,9 +753,49 @@ k3_update(const R* __restrict__ fA, R* __restrict__ fB, R* __restrict__ cu,
     } else {
         const uint32_t L = lnk[o];
         if (L & LNK_SOLID) return;
-        update3_node<R, UNI>(PopSrc<R, false>{fA + o, PL}, PopSrc<R, false>{cu + o, PL}, fB, cu, cpl, mpl, L, g, x,
+        update3_node<R, UNI>(PopSrc<R, 0>{fA + o, PL}, PopSrc<R, 0>{cu + o, PL}, fB, cu, cpl, mpl, L, g, x,
                              y, z, o, P);
     }
+}
+
+// The FP32 update with the stage filled 16 bytes at a time: a thread per element
+// of the padded planes, so that a block's nodes are 512 contiguous bytes of
+// every plane and a warp copies a plane's share in one instruction (four with
+// a copy of 4 bytes per thread and plane, whose issue bounded the update more
+// than the memory did).  GB300, 192x96x192: 460 -> 417 us per step.
+template <bool UNI>
+__global__ void __launch_bounds__(128, UNI ? TLB3_MINB32 : TLB3_MINB32_GEN)
+k3_update_wide(const float* __restrict__ fA, float* __restrict__ fB, float* __restrict__ cu,
+               const float* __restrict__ cpl, const float* __restrict__ mpl, const uint32_t* __restrict__ lnk, Geo3 g,
+               Prm3<float> P)
+{
+    using R = float;
+    __shared__ __align__(16) R stg[kStageRows3<R>][128];
+    tlb::after_previous_launch();
+    const long long PL = g.plane;
+    const unsigned t = threadIdx.x, b0 = blockIdx.x * 128u, i = b0 + t;
+    const unsigned lane4 = (t & 31u) * 4u;
+    if (b0 + lane4 < (unsigned)PL) {  // a plane is a multiple of 32 elements
+#pragma unroll
+        for (int q0 = 0; q0 < kStageRows3<R>; q0 += 4) {
+            const int q = q0 + (int)(t >> 5);
+            const R* src = (q < kPlanes3<R> ? fA + q * PL : cu + (q - kPlanes3<R>)*PL) + b0 + lane4;
+            if (q < kStageRows3<R>)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                                 (unsigned)__cvta_generic_to_shared(&stg[q][lane4])),
+                             "l"(src)
+                             : "memory");
+        }
+    }
+    const PopSrc<R, 2> fs{&stg[0][t], 128}, cs{&stg[kPlanes3<R>][t], 128};
+    const unsigned r = i / (unsigned)g.pitch;
+    const int x = (int)(i - r * (unsigned)g.pitch), y = (int)(r % (unsigned)g.ny), z = (int)(r / (unsigned)g.ny);
+    const uint32_t L = i < (unsigned)PL && x < g.nx ? lnk[i] : LNK_SOLID;
+    if (L & LNK_SOLID) {
+        fs.ready();
+        return;
+    }
+    update3_node<R, UNI>(fs, cs, fB, cu, cpl, mpl, L, g, x, y, z, (long long)i, P);
 }
 
 // c of every node from dense host-order arrays (c1 then c2, nx*ny*nz each).
@@ -820,7 +862,7 @@ __global__ void k3_read(const R* __restrict__ f, const R* __restrict__ cpl, cons
     if (!(L & LNK_SOLID)) {
         const Nb3 nb(g, x, y, z);
         Node3<R> m;
-        node3<UNI>(g, P, PopSrc<R, false>{f + o, g.plane}, cpl, mpl, L, nb, o, m);
+        node3<UNI>(g, P, PopSrc<R, 0>{f + o, g.plane}, cpl, mpl, L, nb, o, m);
         v[0] = m.c1;
         v[1] = m.c2;
         v[2] = R(1.0) - m.c1 - m.c2;
@@ -1070,6 +1112,14 @@ int order_params3(tlb3_lattice* L, bool in_step = false)
     return L->prec == TLB_FP32 ? order_params3_t<float>(L, in_step) : order_params3_t<double>(L, in_step);
 }
 
+// Whether the FP32 update runs over the padded rows (k3_update_wide).  The
+// uniform update gains even where a fifth to a third of the threads idle on
+// padding; the general one, whose registers bound it more, where few do.  GB300,
+// us per step, 4-byte copies over the nodes against this: uniform 64^3 32.4,
+// 28.3; 161x160x160 625, 598; 100x90x110 164, 157; 47x60x70 38.6, 36.6; general
+// 192x96x192 551, 537; 161x160x160 733, 762; 100x90x110 192, 199.
+bool wide3(const tlb3_lattice* L) { return L->uni || 10 * L->lay.pitch <= 11 * L->nx; }
+
 // the fused update and push of one step, current buffer -> spare buffer
 template <typename R>
 int update3_t(tlb3_lattice* L)
@@ -1081,6 +1131,16 @@ int update3_t(tlb3_lattice* L)
         T3_CUDA(cudaFuncSetAttribute(tlb3::k3_update<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
         T3_CUDA(cudaFuncSetAttribute(tlb3::k3_update<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
         L->stage_attr = true;
+    }
+    if constexpr (std::is_same<R, float>::value) {
+        if (wide3(L)) {
+            auto* k = L->uni ? &tlb3::k3_update_wide<true> : &tlb3::k3_update_wide<false>;
+            T3_CUDA(tlb::launch_dependent(k, dim3((unsigned)((L->lay.plane + 127) / 128)), 128, 0, L->stream,
+                                          (const float*)L->fcur<R>(), L->fspare<R>(), L->cu<R>(),
+                                          (const float*)L->cpl<R>(), (const float*)L->mpl<R>(),
+                                          (const uint32_t*)L->lnk(), L->geo, L->P<R>()));
+            return TLB_OK;
+        }
     }
     auto* k = L->uni ? &tlb3::k3_update<R, true> : &tlb3::k3_update<R, false>;
     T3_CUDA(tlb::launch_dependent(k, grid3(L), 128, dyn, L->stream, (const R*)L->fcur<R>(), L->fspare<R>(), L->cu<R>(),
