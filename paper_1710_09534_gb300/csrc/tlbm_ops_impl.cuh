@@ -5,6 +5,7 @@
 #include "tlbm_kernels.cuh"
 #include "tlbm_ops.h"
 #include "tlbm_tile.cuh"
+#include <cmath>
 
 namespace tlb {
 
@@ -100,18 +101,29 @@ inline int sm_count()
 #ifndef TLB_ADAPTIVE_ROWS
 #define TLB_ADAPTIVE_ROWS 1
 #endif
-// one_wave (the FP64 two-buffer interior kernel): a lattice large enough for
+// one_wave (the FP64 interior kernels): a lattice large enough for
 // more than one wave of blocks gets segments long enough that the whole grid
 // is resident at once, so that the halo rows' c sums and chemical potentials
 // (FP64 arithmetic, the kernel's bound) are repeated on fewer rows.  GB300:
 // FP64 2048^2 interior kernel 1.929 -> 1.911 ms, 1024x2048 cylinder impact
 // within +-3%.  FP32 and 16-bit storage (latency-bound) lose the dynamic
 // balancing of several waves: the cylinder impact ran 12% (FP32) and 10%
-// (FP16) slower, so they keep short segments; the in-place kernels too.
+// (FP16) slower, so they keep short segments.
 #ifndef TLB_ONE_WAVE
 #define TLB_ONE_WAVE 1
 #endif
-inline int rows_for(const Geo& g, int tx, int rows, int per_sm, bool one_wave = false)
+// Otherwise segments of 12 to 24 rows, of the length that wastes least: blocks
+// come in waves of the resident ones, so w = blocks / resident of them last
+// ceil(w) / w as long as full waves would, and the `halo` rows' loads are
+// repeated per segment (16 rows unless another length saves 2%; halo = 0: no
+// such choice).  GB300, us per step, 16 rows against this: FP32 2048^2 204.5,
+// 201.9; 1800x1700 154.5, 149.5; 3000x2000 300, 292; FP16 1500x1300 88.0, 77.6;
+// 1800x1700 119.6, 110.6; 1024x2048 impact 91.5, 87.4; in place FP32 2048x1024
+// 168.5, 152.7; 1500x1300 165, 152.  In place with 16-bit storage it lost as
+// often as it gained (2048x1024 123.6, 126.0; 2048^2 237.6, 231.5) and is off.
+// In-place FP64 takes the one-wave rule, in which its halo is cheap (c comes
+// from planes): 2048x1024 1016 -> 889.
+inline int rows_for(const Geo& g, int tx, int rows, int per_sm, bool one_wave, int halo)
 {
     if (!TLB_ADAPTIVE_ROWS) return rows;
     const int strips = (g.nx + tx - 1) / tx;
@@ -122,7 +134,19 @@ inline int rows_for(const Geo& g, int tx, int rows, int per_sm, bool one_wave = 
             if (r > rows) return r;
         }
     }
-    while (rows > 4 && (long long)strips * ((g.ny + rows - 1) / rows) < (long long)sm_count() * per_sm) rows /= 2;
+    const long long slots = (long long)sm_count() * per_sm;
+    auto blocks = [&](int r) { return (long long)strips * ((g.ny + r - 1) / r); };
+    if (halo > 0 && blocks(rows) >= slots) {
+        auto cost = [&](int r) {
+            const double w = (double)blocks(r) / slots;
+            return std::ceil(w) / w * (r + halo) / r;
+        };
+        int best = rows;
+        for (int r = 12; r <= 24; r++)
+            if (cost(r) < 0.98 * cost(rows) && cost(r) < cost(best)) best = r;
+        return best;
+    }
+    while (rows > 4 && blocks(rows) < slots) rows /= 2;
     return rows;
 }
 
@@ -144,7 +168,7 @@ struct OpsImpl {
         static_assert(BLOCK == 32 * kWallTY, "a block takes a strip segment or a near-wall tile");
         // equal densities and viscosities: the uniform-property update
         const bool uni = Pd.uni != 0.0;
-        const int rows = rows_for(g, TX, ROWS, uni ? kMinBUni : MINB, std::is_same<R, double>::value);
+        const int rows = rows_for(g, TX, ROWS, uni ? kMinBUni : MINB, std::is_same<R, double>::value, 4);
         const int strips = (g.nx + TX - 1) / TX, segs = (g.ny + rows - 1) / rows;
         auto* k = uni ? &k_step_march<S, R, BLOCK, PREFETCH, kMinBUni, MRT, true>
                       : &k_step_march<S, R, BLOCK, PREFETCH, MINB, MRT, false>;
@@ -313,7 +337,7 @@ struct OpsImpl {
     {
         constexpr int TX = BLOCK - 4;
         constexpr int kMinB = ODD ? kMinBIpOdd : kMinBIpEven;
-        const int rows = rows_for(g, TX, ROWS, kMinB);
+        const int rows = rows_for(g, TX, ROWS, kMinB, std::is_same<R, double>::value, Store<S>::k16 ? 0 : 1);
         dim3 grid((g.nx + TX - 1) / TX, (g.ny + rows - 1) / rows);
         k_step_interior_ip<S, R, BLOCK, ROWS, PREFETCH, kMinB, MRT, UNI, ODD><<<grid, BLOCK, 0, s>>>(
             (S*)f, (CuT<S>*)cu, (const R*)cpl, cls, g, P, rows);
