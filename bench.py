@@ -1,8 +1,8 @@
 #!/usr/bin/env python
 """Throughput of the ternary phase-field lattice Boltzmann update on GB300.
 
-One bench step = one time step of the whole hot path (fused interior kernel +
-near-wall kernel) over the 2048x2048 tiled-drops lattice (binary drops on a
+One bench step = one time step of the whole hot path (fused interior update and
+near-wall nodes in one launch) over the 2048x2048 tiled-drops lattice (binary drops on a
 wetting bottom wall, neutral top wall, periodic in x, free compound drops in
 the bulk).  The state (FP64: 1.8 GB double-buffered) is far larger than the
 129 MB L2, so no explicit flush is needed between steps.
@@ -58,8 +58,8 @@ def storage_bytes_per_node(precision):
     return 2 * (25 * 2 + 4 * 4 + 4 * 4)
 
 
-KERNEL = {"fp64": "k_step_march<double>", "fp32": "k_step_interior<float>",
-          "fp16": "k_step_march<__half>", "bf16": "k_step_interior<__nv_bfloat16>"}
+KERNEL = {"fp64": "k_step_march<double>", "fp32": "k_step_march<float>",
+          "fp16": "k_step_march<__half>", "bf16": "k_step_march<__nv_bfloat16>"}
 
 
 # FP64 arithmetic per node update of the fused interior kernel as counted by
@@ -67,11 +67,11 @@ KERNEL = {"fp64": "k_step_march<double>", "fp32": "k_step_interior<float>",
 # FMA as 2).  "uniform": the update taken when all three fluids share density
 # and viscosity (the tiled-drops workload); "general": any densities and
 # viscosities (the same lattice with rho_2 = 3).
-FP64_DP = {"uniform": (216.9, 312.9), "general": (281.1, 407.4)}
+FP64_DP = {"uniform": (204.5, 297.4), "general": (267.0, 390.2)}
 # The same counts for the D3Q19 update kernel k3_update (ncu, 128x64x128
-# drops on a wetting wall, uniform properties: 150.0 DFMA + 149.0 DADD + 53.0
+# drops on a wetting wall, uniform properties: 147.0 DFMA + 143.0 DADD + 50.0
 # DMUL per node).
-FP64_DP3 = {"uniform": (352.0, 502.0)}
+FP64_DP3 = {"uniform": (340.0, 487.0)}
 # FP64 vector unit: 152 SMs x 2 DP instructions/clk x 2.07 GHz (an FMA is 2 flops)
 FP64_DP_INST_PEAK = 152 * 2 * 2.07e9
 FP64_PEAK_TFLOPS = 2 * FP64_DP_INST_PEAK / 1e12
@@ -437,9 +437,9 @@ def run_ours(args):
         "hbm_roofline_pct": round(100 * mlups / ws * 1e6 * bytes_node / (hbm_gbs * 1e9), 2),
         "roofline": roof,
         "kernel_ms": {"interior_avg": round(k1_avg, 4), "wall_avg": round(k2_ms / max(k2_n, 1), 4),
-                      "wall_note": "the near-wall kernel runs on a side stream concurrently with the interior "
-                                   "kernel; its time spans launch to end, mostly waiting for SMs"},
-        # two buffers: interior + near-wall kernel per step; in place: the
+                      "wall_note": "two buffers: the near-wall tiles are blocks of the interior launch; in place: a "
+                                   "kernel on a side stream, whose time spans launch to end"},
+        # two buffers: one launch per step; in place: the
         # order-parameter pass, the interior, the lid row (if any) and the
         # near-wall kernel, plus the streaming swap after an odd step count
         "gpu_launches": int(k1_n + k2_n) if not args.inplace else

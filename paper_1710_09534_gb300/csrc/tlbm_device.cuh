@@ -119,8 +119,9 @@ __device__ __forceinline__ int site_of(const Geo& g, const uint8_t* __restrict__
 __device__ __forceinline__ bool fluidlike(int s) { return s == ST_FLUID || s == ST_LID; }
 
 // FP64 arithmetic, whose instructions bound its kernels, takes forms of the
-// same terms with fewer of them (uniform-property update 168 -> 154, mu 23 -> 21
-// per node; of the same accuracy, in a different rounding):
+// same terms with fewer of them (216.9 -> 204.5 per node of the uniform-property
+// marching kernel, 281.1 -> 267.0 of the general one, ncu; of the same accuracy,
+// in a different rounding):
 //   Q_i     kq c u + ks (c u - old) = (kq + ks) c u - ks old
 //   a       4.5 (e.u)^2 - 1.5 u.u from u_x^2, u_y^2 and the product 9 u_x u_y
 //   R_X, P_X of the diagonal links = 1/4 of those of the axis links
