@@ -8,7 +8,7 @@
 //                    local), mu_1, mu_2 on the tile plus radius 1 in shared
 //                    memory, then the per-node update.
 //                    (the other fluid nodes: tlbm_tile.cuh)
-//   k_init, k_read_fields, k_mass_partials/k_mass_final
+//   k_init, k_mass_partials/k_mass_final
 #pragma once
 #include <type_traits>
 #include <cuda_bf16.h>
@@ -1041,16 +1041,6 @@ __device__ __forceinline__ void window_macros(const Geo& g, const uint8_t* __res
     m.rho = density(P, m.c1, m.c2);
 }
 
-template <typename S, typename R>
-struct DistFetch {
-    const S* f;
-    long long PL;
-    __device__ __forceinline__ void operator()(long long off, R& a, R& b) const
-    {
-        order_params<R>(f, PL, off, a, b);
-    }
-};
-
 // c_1, c_2 from dense FP64 row arrays holding rows y_b .. y_b + rows - 1 of
 // the lattice (y_b may be negative; rows outside 0 .. ny-1 hold the wrapped
 // rows of a periodic y axis); the whole lattice is y_b = 0, rows = ny.
@@ -1126,57 +1116,6 @@ __global__ void k_init(S* __restrict__ fA, CuT<S>* __restrict__ cu, const uint8_
     cu[1 * PL + o] = CuT<S>(m.c1 * v);
     cu[2 * PL + o] = CuT<S>(m.c2 * u);
     cu[3 * PL + o] = CuT<S>(m.c2 * v);
-}
-
-// ---------------------------------------------------------------------------
-// Read-out of macroscopic fields as FP64 planes (order c1 c2 c3 rho ux uy p
-// mu1 mu2 mu3, only the planes selected by `mask`).
-// ---------------------------------------------------------------------------
-template <typename S, typename R>
-__global__ void k_read_fields(const S* __restrict__ fA, const uint8_t* __restrict__ cls, double* __restrict__ out,
-                              uint32_t mask, Geo g, Prm<R> P)
-{
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y;
-    if (x >= g.nx) return;
-    const long long PL = g.plane;
-    const long long o = (long long)y * g.pitch + x;
-    const long long n = (long long)y * g.nx + x;
-    const long long N = (long long)g.nx * g.ny;
-    const int kind = cls[o] & CLS_KIND_MASK;
-    double v[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-    if (fluidlike(kind)) {
-        DistFetch<S, R> fetch{fA, PL};
-        const long long of = kind == ST_LID ? o - g.pitch : o;
-        Macro<R> m;
-        window_macros(g, cls, P, x, kind == ST_LID ? y - 1 : y, fetch, m);
-        R gv[9];
-        for (int k = 0; k < 9; k++) gv[k] = ld_pop<R>(fA, 18 + k, PL, of);
-        Hydro<R> h;
-        hydro_from_g(P, m, gv, h);
-        if (kind == ST_LID) {
-            h.ux = P.lid_u;
-            h.uy = R(0);
-        }
-        const R mu3 = -fma(P.l3_l1, m.mu1, P.l3_l2 * m.mu2);
-        v[0] = m.c1;
-        v[1] = m.c2;
-        v[2] = R(1) - m.c1 - m.c2;
-        v[3] = m.rho;
-        v[4] = h.ux;
-        v[5] = h.uy;
-        v[6] = h.p;
-        v[7] = m.mu1;
-        v[8] = m.mu2;
-        v[9] = mu3;
-    }
-    int plane = 0;
-    for (int q = 0; q < 10; q++) {
-        if (mask & (1u << q)) {
-            out[plane * N + n] = v[q];
-            plane++;
-        }
-    }
 }
 
 // ---------------------------------------------------------------------------

@@ -232,8 +232,10 @@ struct OpsImpl {
                             const Prm<double>& Pd, cudaStream_t s)
     {
         const Prm<R> P = cast_prm<R>(Pd);
-        dim3 grid((g.nx + 127) / 128, g.ny);
-        k_read_fields<S, R><<<grid, 128, 0, s>>>((const S*)fA, cls, out, mask, g, P);
+        constexpr int TY = 8;
+        const int shift = tile_shift(g.edge[3] == EDGE_LID, g.ny, TY);
+        dim3 grid((g.nx + 31) / 32, (g.ny + shift + TY - 1) / TY);
+        k_read_fields<S, R, TY><<<grid, 32 * TY, 0, s>>>((const S*)fA, cls, out, mask, g, P, shift);
         return cudaGetLastError();
     }
     static cudaError_t mass(const void* fA, const uint8_t* cls, double* part, int nparts, double* out,
