@@ -229,8 +229,7 @@ __global__ void k3_links(const uint8_t* __restrict__ kind, uint32_t* __restrict_
 
 // c_1, c_2 of every node (Eq. 13a); zero on solids.
 template <typename R>
-__global__ void k3_csum(const R* __restrict__ f, R* __restrict__ cpl, const uint8_t* __restrict__ kind,
-                        Geo3 g)
+__global__ void k3_csum(const R* f, R* cpl, const uint8_t* __restrict__ kind, Geo3 g)
 {
     tlb::after_previous_launch();
     NODE_OF_THREAD
@@ -279,8 +278,7 @@ __device__ __forceinline__ void mu_from_sums(const Prm3<R>& P, uint32_t L, R c1,
 
 // mu_1, mu_2 of every fluid node (zero on solids).
 template <typename R>
-__global__ void k3_mu(const R* __restrict__ cpl, R* __restrict__ mpl, const uint32_t* __restrict__ lnk,
-                      Geo3 g, Prm3<R> P)
+__global__ void k3_mu(const R* cpl, R* mpl, const uint32_t* __restrict__ lnk, Geo3 g, Prm3<R> P)
 {
     tlb::after_previous_launch();
     NODE_OF_THREAD
@@ -718,8 +716,7 @@ __device__ __forceinline__ void update3_node(const PopSrc<R, STG>& fs, const Pop
 
 template <typename R, bool UNI>
 __global__ void __launch_bounds__(128, kLo3<R> ? (UNI ? TLB3_MINB32 : TLB3_MINB32_GEN) : (UNI ? TLB3_MINB : TLB3_MINB_GEN))
-k3_update(const R* __restrict__ fA, R* __restrict__ fB, R* __restrict__ cu,
-          const R* __restrict__ cpl, const R* __restrict__ mpl, const uint32_t* __restrict__ lnk, Geo3 g,
+k3_update(const R* fA, R* fB, R* cu, const R* cpl, const R* mpl, const uint32_t* __restrict__ lnk, Geo3 g,
           Prm3<R> P)
 {
     tlb::after_previous_launch();
@@ -765,9 +762,8 @@ k3_update(const R* __restrict__ fA, R* __restrict__ fB, R* __restrict__ cu,
 // than the memory did).  GB300, 192x96x192: 460 -> 417 us per step.
 template <bool UNI>
 __global__ void __launch_bounds__(128, UNI ? TLB3_MINB32 : TLB3_MINB32_GEN)
-k3_update_wide(const float* __restrict__ fA, float* __restrict__ fB, float* __restrict__ cu,
-               const float* __restrict__ cpl, const float* __restrict__ mpl, const uint32_t* __restrict__ lnk, Geo3 g,
-               Prm3<float> P)
+k3_update_wide(const float* fA, float* fB, float* cu, const float* cpl, const float* mpl,
+               const uint32_t* __restrict__ lnk, Geo3 g, Prm3<float> P)
 {
     using R = float;
     __shared__ __align__(16) R stg[kStageRows3<R>][128];

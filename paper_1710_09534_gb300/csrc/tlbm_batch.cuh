@@ -52,7 +52,7 @@ struct BatchCounters {
 template <typename S, typename R, int BLOCK, bool PREFETCH, int MINB, bool MRT>
 __global__ void __launch_bounds__(BLOCK, MINB)
 k_batch_interior(const LatDesc<R>* __restrict__ descs, const TileItem* __restrict__ items,
-                 const WallItem* __restrict__ walls, BatchCounters* __restrict__ ctr, int parity)
+                 const WallItem* __restrict__ walls, BatchCounters* ctr, int parity)
 {
     constexpr int WTY = BLOCK / 32;
     constexpr bool kStash = kStashPops && std::is_same<R, float>::value && !kDenseMrt<S, MRT>;
@@ -77,9 +77,9 @@ k_batch_interior(const LatDesc<R>* __restrict__ descs, const TileItem* __restric
             reinterpret_cast<R*>(&Ps)[i] = reinterpret_cast<const R*>(&d->P)[i];
         __syncthreads();
         const Geo g = d->g;
-        const S* fA = (const S*)d->buf[parity];
-        S* fB = (S*)d->buf[parity ^ 1];
-        CuT<S>* cu = (CuT<S>*)d->cu;
+        const S* fA = global_ptr((const S*)d->buf[parity]);
+        S* fB = global_ptr((S*)d->buf[parity ^ 1]);
+        CuT<S>* cu = global_ptr((CuT<S>*)d->cu);
         // members with equal densities and viscosities take the uniform-property
         // update, as they do when stepped alone (the branch is uniform per tile)
         auto* st = reinterpret_cast<PopStash<R, BLOCK>*>(&sh.m.stash);  // used only when kStash

@@ -740,10 +740,26 @@ struct MrtNode {
 // while the launch before them in the stream finishes; after_previous_launch
 // waits until that one is complete and lets the next one start its blocks.
 // What a kernel reads before it must not be written by an earlier step.
+//
+// Such a block is resident while the launch before it still writes.  So what any
+// step writes is read by plain loads, not through the read-only path (__ldg, or
+// a load of a const __restrict__ kernel argument, which the compiler turns into
+// one): griddepcontrol.wait orders only the former.  For the same reason these
+// kernels' pointers to it carry no __restrict__: a load through one could be
+// moved above the wait, since the memory clobber does not cover memory that
+// nothing else may reach.
 __device__ __forceinline__ void after_previous_launch()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+// A pointer that was itself read from memory, or passed to a call, as one to
+// global memory.
+template <typename T>
+__device__ __forceinline__ T* global_ptr(T* p)
+{
+    __builtin_assume(__isGlobal(p));
+    return p;
 }
 template <typename K, typename... A>
 inline cudaError_t launch_dependent(K k, dim3 grid, int threads, size_t shared, cudaStream_t s, A... args)

@@ -137,8 +137,10 @@ __device__ __forceinline__ long long idx16(int q, long long PL, long long o)
     return 16 * PL + (long long)(q - 18) * PL + o;
 }
 
-// Load through the read-only path (NC: the buffer is not written during the
-// kernel) or a plain coherent load (the in-place update writes what it reads).
+// Load through the read-only path (NC: nothing writes the buffer while the
+// kernel is resident) or a plain coherent load (the in-place update writes what
+// it reads; a dependent launch is resident while the launch before it still
+// writes, see after_previous_launch).
 template <bool NC, typename T>
 __device__ __forceinline__ T ld_any(const T* p)
 {
@@ -257,15 +259,15 @@ __device__ __forceinline__ void st_three(S* __restrict__ f, int k, long long PL,
 }
 
 // c_i = sum_k f^i_k of node o for i = 1, 2 (rest population hi + lo)
-template <typename R, typename S>
+template <typename R, bool NC = true, typename S>
 __device__ __forceinline__ void order_params(const S* __restrict__ f, long long PL, long long o, R& c1, R& c2)
 {
     R v[18];
 #pragma unroll
-    for (int k = 0; k < 18; k++) v[k] = ld_pop<R>(f, k, PL, o);
+    for (int k = 0; k < 18; k++) v[k] = ld_pop<R, NC>(f, k, PL, o);
     if constexpr (Store<S>::kLo) {
-        v[0] += ld_lo<R>(f, 0, PL, o);
-        v[9] += ld_lo<R>(f, 1, PL, o);
+        v[0] += ld_lo<R, NC>(f, 0, PL, o);
+        v[9] += ld_lo<R, NC>(f, 1, PL, o);
     }
     c1 = sum9(v);
     c2 = sum9(v + 9);
@@ -605,6 +607,14 @@ constexpr bool kPipeRows16 = TLB_PIPE16R != 0;
 // iteration's update row are loaded one iteration ahead as well (as stored,
 // 13 registers): 16-bit storage, GB300, 2048^2, 5 blocks per SM: FP16 25.3 ->
 // 26.1, BF16 26.6 -> 27.2 G node updates/s.
+// Where an iteration issues these loads matters since they are plain ones, which
+// the compiler moves over no barrier: it decides what is live in the phases
+// between, at 96 registers.  GB300, us per step, all at the top of the iteration
+// against this (g and c_i u at the update; the c row after the first barrier in
+// the uniform update, at the top in the general one): FP16 2048^2 155.8, 142.4;
+// 1500x1300 80.9, 73.4; 1024x2048 impact (general) 88.7, 87.7, and 105.6 with its
+// c row after the barrier too; BF16 2048^2 152.0, 144.1.  Through the read-only
+// path, without the overlap of launches: 149.5, 78.0, 97.7, 155.0.
 #ifndef TLB_PIPEG16
 #define TLB_PIPEG16 1
 #endif
@@ -623,7 +633,7 @@ struct Raw16Row {
 
 // One tile: strip bx (columns bx*(BLOCK-4) .. +BLOCK-5), segment by (rows
 // by*rows .. +rows-1, marching up for even by and down for odd by).
-template <typename S, typename R, int BLOCK, bool PREFETCH, bool MRT, bool UNI = false, bool STASH = false>
+template <typename S, typename R, int BLOCK, bool PREFETCH, bool MRT, bool UNI, bool STASH>
 __device__ __forceinline__ void interior_tile(const S* __restrict__ fA, S* __restrict__ fB, CuT<S>* __restrict__ cu,
                                               const uint8_t* __restrict__ cls, const Geo& g, const Prm<R>& P,
                                               int bx, int by, int rows, ColRings<R, BLOCK>& sh,
@@ -666,12 +676,12 @@ __device__ __forceinline__ void interior_tile(const S* __restrict__ fA, S* __res
         }
         if (in) {
             const long long oc = (long long)yw * g.pitch + xw;
-            v[0] = ld_pop<R>(fA, 0, PL, oc);
-            v[9] = ld_pop<R>(fA, 9, PL, oc);
+            v[0] = ld_pop<R, false>(fA, 0, PL, oc);
+            v[9] = ld_pop<R, false>(fA, 9, PL, oc);
 #pragma unroll
-            for (int k = 1; k < 9; k++) ld_pair<R, true, SE != 0>(fA, k, PL, oc, v[k], v[9 + k]);
-            l[0] = ld_lo<R>(fA, 0, PL, oc);
-            l[1] = ld_lo<R>(fA, 1, PL, oc);
+            for (int k = 1; k < 9; k++) ld_pair<R, false, SE != 0>(fA, k, PL, oc, v[k], v[9 + k]);
+            l[0] = ld_lo<R, false>(fA, 0, PL, oc);
+            l[1] = ld_lo<R, false>(fA, 1, PL, oc);
         } else {
 #pragma unroll
             for (int k = 0; k < 18; k++) v[k] = R(0);
@@ -692,12 +702,12 @@ __device__ __forceinline__ void interior_tile(const S* __restrict__ fA, S* __res
             const long long oc = (long long)yw * g.pitch + xw;
             const unsigned* wp = reinterpret_cast<const unsigned*>(fA);
 #pragma unroll
-            for (int k = 0; k < 8; k++) q.w[k] = __ldg(wp + (long long)k * PL + oc);
+            for (int k = 0; k < 8; k++) q.w[k] = wp[(long long)k * PL + oc];
             const float* rp = rest_region(fA, PL);
 #pragma unroll
             for (int i = 0; i < 2; i++) {
-                q.r[i] = __ldg(rp + i * PL + oc);
-                q.l[i] = __ldg(rp + (2 + i) * PL + oc);
+                q.r[i] = rp[i * PL + oc];
+                q.l[i] = rp[(2 + i) * PL + oc];
             }
         } else {
 #pragma unroll
@@ -738,7 +748,7 @@ __device__ __forceinline__ void interior_tile(const S* __restrict__ fA, S* __res
                 cl[0] = R(nq.l[0]);
                 cl[1] = R(nq.l[1]);
             }
-            if (it + 1 < iters) load_raw_row(yc + dir, nq);
+            if (!UNI && it + 1 < iters) load_raw_row(yc + dir, nq);
         }
         // the update node (row yu of this column, if any): its g and c_i u
         // are the first touches of HBM, issued before its node class is
@@ -749,34 +759,9 @@ __device__ __forceinline__ void interior_tile(const S* __restrict__ fA, S* __res
         const long long ou = in_rows ? (long long)yu * g.pitch + xs : 0;
         const bool upd = in_rows && (cls[ou] & CLS_INTERIOR) != 0;
         R gv[9], cp[4];
-        if constexpr (PIPEG) {
-            if constexpr (Store<S>::k16) {
-                constexpr float inv = SE != 0 ? 1.0f : 1.0f / float(1 << Store<S>::kScaleExp);
+        if (!PIPEG && PREFETCH && in_rows) {
 #pragma unroll
-                for (int k = 0; k < 9; k++) gv[k] = R(dec16(S{}, ngr[k]) * inv);
-            } else {
-#pragma unroll
-                for (int k = 0; k < 9; k++) gv[k] = R(ngr[k]);
-            }
-#pragma unroll
-            for (int q = 0; q < 4; q++) cp[q] = R(ncp[q]);
-            // the next iteration's update row (yu + dir), if it has one
-            if (updater && it + 1 >= 4 && it + 1 < iters) {
-                const long long on = (long long)(yu + dir) * g.pitch + xs;
-                if constexpr (Store<S>::k16) {
-                    const unsigned short* gp = reinterpret_cast<const unsigned short*>(fA);
-#pragma unroll
-                    for (int k = 0; k < 9; k++) ngr[k] = __ldg(gp + idx16(18 + k, PL, on));
-                } else {
-#pragma unroll
-                    for (int k = 0; k < 9; k++) ngr[k] = __ldg(fA + (18 + k) * PL + on);
-                }
-#pragma unroll
-                for (int q = 0; q < 4; q++) ncp[q] = __ldg(&cu[q * PL + on]);
-            }
-        } else if (PREFETCH && in_rows) {
-#pragma unroll
-            for (int k = 0; k < 9; k++) gv[k] = ld_pop<R, true, SE != 0>(fA, 18 + k, PL, ou);
+            for (int k = 0; k < 9; k++) gv[k] = ld_pop<R, false, SE != 0>(fA, 18 + k, PL, ou);
 #pragma unroll
             for (int q = 0; q < 4; q++) cp[q] = R(cu[q * PL + ou]);
         }
@@ -799,12 +784,12 @@ __device__ __forceinline__ void interior_tile(const S* __restrict__ fA, S* __res
                         l1 = cl[0];
                         l2 = cl[1];
                     } else {
-                        v[0] = ld_pop<R>(fA, 0, PL, oc);
-                        v[9] = ld_pop<R>(fA, 9, PL, oc);
+                        v[0] = ld_pop<R, false>(fA, 0, PL, oc);
+                        v[9] = ld_pop<R, false>(fA, 9, PL, oc);
 #pragma unroll
-                        for (int k = 1; k < 9; k++) ld_pair<R, true, SE != 0>(fA, k, PL, oc, v[k], v[9 + k]);
-                        l1 = ld_lo<R>(fA, 0, PL, oc);
-                        l2 = ld_lo<R>(fA, 1, PL, oc);
+                        for (int k = 1; k < 9; k++) ld_pair<R, false, SE != 0>(fA, k, PL, oc, v[k], v[9 + k]);
+                        l1 = ld_lo<R, false>(fA, 0, PL, oc);
+                        l2 = ld_lo<R, false>(fA, 1, PL, oc);
                     }
                     float4(&st)[5][BLOCK] = stash->v[(yc + 9) % 3];
                     static_for<0, 4>([&](auto pc) {
@@ -817,7 +802,7 @@ __device__ __forceinline__ void interior_tile(const S* __restrict__ fA, S* __res
                     a = sum9s<SE>(v);
                     b = sum9s<SE>(v + 9);
                 } else {
-                    order_params<R>(fA, PL, oc, a, b);
+                    order_params<R, false>(fA, PL, oc, a, b);
                 }
             }
             ca[2] = ca[1];
@@ -835,6 +820,9 @@ __device__ __forceinline__ void interior_tile(const S* __restrict__ fA, S* __res
             }
         }
         __syncthreads();
+        if constexpr (PIPE16 && UNI) {  // (see kPipeG16)
+            if (it + 1 < iters) load_raw_row(yc + dir, nq);
+        }
         // 2) mu of row ym (Eq. 8 with Eq. 20b)
         if (it >= 2 && t >= 1 && t < BLOCK - 1) {
             const int sl = (ym + 9) % 3;
@@ -861,6 +849,32 @@ __device__ __forceinline__ void interior_tile(const S* __restrict__ fA, S* __res
         // the barrier)
         __syncthreads();
         // 3) update of row yu
+        if constexpr (PIPEG) {
+            if constexpr (Store<S>::k16) {
+                constexpr float inv = SE != 0 ? 1.0f : 1.0f / float(1 << Store<S>::kScaleExp);
+#pragma unroll
+                for (int k = 0; k < 9; k++) gv[k] = R(dec16(S{}, ngr[k]) * inv);
+            } else {
+#pragma unroll
+                for (int k = 0; k < 9; k++) gv[k] = R(ngr[k]);
+            }
+#pragma unroll
+            for (int q = 0; q < 4; q++) cp[q] = R(ncp[q]);
+            // the next iteration's update row (yu + dir), if it has one
+            if (updater && it + 1 >= 4 && it + 1 < iters) {
+                const long long on = (long long)(yu + dir) * g.pitch + xs;
+                if constexpr (Store<S>::k16) {
+                    const unsigned short* gp = reinterpret_cast<const unsigned short*>(fA);
+#pragma unroll
+                    for (int k = 0; k < 9; k++) ngr[k] = gp[idx16(18 + k, PL, on)];
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 9; k++) ngr[k] = fA[(18 + k) * PL + on];
+                }
+#pragma unroll
+                for (int q = 0; q < 4; q++) ncp[q] = cu[q * PL + on];
+            }
+        }
         if (!upd) continue;
         Macro<R> m;
         {
@@ -887,7 +901,7 @@ __device__ __forceinline__ void interior_tile(const S* __restrict__ fA, S* __res
         }
         if (!PREFETCH) {
 #pragma unroll
-            for (int k = 0; k < 9; k++) gv[k] = ld_pop<R, true, SE != 0>(fA, 18 + k, PL, ou);
+            for (int k = 0; k < 9; k++) gv[k] = ld_pop<R, false, SE != 0>(fA, 18 + k, PL, ou);
 #pragma unroll
             for (int q = 0; q < 4; q++) cp[q] = R(cu[q * PL + ou]);
         }
@@ -912,10 +926,10 @@ __device__ __forceinline__ void interior_tile(const S* __restrict__ fA, S* __res
                     f2k = stash_hi(K) ? sv.w : sv.y;
                 } else {
                     if constexpr (K == 0) {
-                        f1k = ld_pop<R>(fA, 0, PL, ou);
-                        f2k = ld_pop<R>(fA, 9, PL, ou);
+                        f1k = ld_pop<R, false>(fA, 0, PL, ou);
+                        f2k = ld_pop<R, false>(fA, 9, PL, ou);
                     } else {
-                        ld_pair<R, true, SE != 0>(fA, K, PL, ou, f1k, f2k);
+                        ld_pair<R, false, SE != 0>(fA, K, PL, ou, f1k, f2k);
                     }
                 }
             },
@@ -925,8 +939,8 @@ __device__ __forceinline__ void interior_tile(const S* __restrict__ fA, S* __res
                     l1 = sv.z;
                     l2 = sv.w;
                 } else {
-                    l1 = ld_lo<R>(fA, 0, PL, ou);
-                    l2 = ld_lo<R>(fA, 1, PL, ou);
+                    l1 = ld_lo<R, false>(fA, 0, PL, ou);
+                    l2 = ld_lo<R, false>(fA, 1, PL, ou);
                 }
             },
             [&](auto kc, auto o1, auto o2, auto og) {

@@ -139,7 +139,7 @@ __device__ __forceinline__ int tile_site(const Geo& g, const uint8_t* __restrict
 // One tile with its first node at (x0, y0).  WALL: its near-wall and lid nodes
 // only (interior nodes lend their c).
 template <typename S, typename R, int TY, bool MRT, bool UNI, bool WALL>
-__device__ __forceinline__ void tile_step(const S* __restrict__ fA, S* __restrict__ fB, CuT<S>* __restrict__ cu,
+__device__ __forceinline__ void tile_step(const S* fA, S* fB, CuT<S>* cu,
                                           const uint8_t* __restrict__ cls, const Geo& g, const Prm<R>& P, int x0,
                                           int y0, TileShared<R, TY>& sh)
 {
@@ -188,15 +188,15 @@ __device__ __forceinline__ void tile_step(const S* __restrict__ fA, S* __restric
     // the thread's own node: everything its update reads, and its c
     R f[18], lo[2] = {R(0), R(0)}, gv[9], cp[4];
     if (own) {
-        f[0] = ld_pop<R>(fA, 0, PL, o);
-        f[9] = ld_pop<R>(fA, 9, PL, o);
+        f[0] = ld_pop<R, false>(fA, 0, PL, o);
+        f[9] = ld_pop<R, false>(fA, 9, PL, o);
 #pragma unroll
-        for (int k = 1; k < 9; k++) ld_pair<R, true, SE != 0>(fA, k, PL, o, f[k], f[9 + k]);
-        lo[0] = ld_lo<R>(fA, 0, PL, o);
-        lo[1] = ld_lo<R>(fA, 1, PL, o);
+        for (int k = 1; k < 9; k++) ld_pair<R, false, SE != 0>(fA, k, PL, o, f[k], f[9 + k]);
+        lo[0] = ld_lo<R, false>(fA, 0, PL, o);
+        lo[1] = ld_lo<R, false>(fA, 1, PL, o);
         if (!WALL || !(mine & CLS_INTERIOR)) {
 #pragma unroll
-            for (int k = 0; k < 9; k++) gv[k] = ld_pop<R, true, SE != 0>(fA, 18 + k, PL, o);
+            for (int k = 0; k < 9; k++) gv[k] = ld_pop<R, false, SE != 0>(fA, 18 + k, PL, o);
 #pragma unroll
             for (int q = 0; q < 4; q++) cp[q] = R(cu[q * PL + o]);
         }
@@ -207,7 +207,7 @@ __device__ __forceinline__ void tile_step(const S* __restrict__ fA, S* __restric
             V c{R(0), R(0)};
             if ((fs[r] & CLS_KIND_MASK) == ST_FLUID) {
                 R a, b;
-                order_params<R>(fA, PL, fo[r], a, b);
+                order_params<R, false>(fA, PL, fo[r], a, b);
                 c = V{a, b};
             }
             sh.c[fj[r]][fi[r]] = c;
@@ -228,7 +228,7 @@ __device__ __forceinline__ void tile_step(const S* __restrict__ fA, S* __restric
                 f[9] = f20;
             } else {
                 R a, b;
-                order_params<R>(fA, PL, oo, a, b);
+                order_params<R, false>(fA, PL, oo, a, b);
                 c = V{a, b};
             }
         }
@@ -348,7 +348,7 @@ __device__ __forceinline__ void tile_step(const S* __restrict__ fA, S* __restric
     const long long of = lid ? o - g.pitch : o;
     if (lid) {
 #pragma unroll
-        for (int k = 0; k < 9; k++) gv[k] = ld_pop<R>(fA, 18 + k, PL, of);
+        for (int k = 0; k < 9; k++) gv[k] = ld_pop<R, false>(fA, 18 + k, PL, of);
     } else if constexpr (SE != 0) {
 #pragma unroll
         for (int k = 0; k < 9; k++) gv[k] *= unscale;
@@ -371,11 +371,11 @@ __device__ __forceinline__ void tile_step(const S* __restrict__ fA, S* __restric
             R e1u, e2u, egu, e1f, e2f, egf;
             equilibria(k, P, m.c1, m.c2, m.mu1, m.mu2, m.rho, h.p, h.ux, h.uy, e1u, e2u, egu);
             equilibria(k, P, m.c1, m.c2, m.mu1, m.mu2, m.rho, h.p, fx, fy, e1f, e2f, egf);
-            R ff1 = ld_pop<R>(fA, k, PL, of), ff2 = ld_pop<R>(fA, 9 + k, PL, of);
+            R ff1 = ld_pop<R, false>(fA, k, PL, of), ff2 = ld_pop<R, false>(fA, 9 + k, PL, of);
             if constexpr (Store<S>::kLo) {
                 if (k == 0) {
-                    ff1 += ld_lo<R>(fA, 0, PL, of);
-                    ff2 += ld_lo<R>(fA, 1, PL, of);
+                    ff1 += ld_lo<R, false>(fA, 0, PL, of);
+                    ff2 += ld_lo<R, false>(fA, 1, PL, of);
                 }
             }
             f[k] = e1u + (ff1 - e1f);
@@ -505,8 +505,7 @@ k_read_fields(const S* __restrict__ fA, const uint8_t* __restrict__ cls, double*
 
 template <typename S, typename R, int TY, int MINB, bool MRT, bool UNI>
 __global__ void __launch_bounds__(32 * TY, MINB)
-k_step_tile(const S* __restrict__ fA, S* __restrict__ fB, CuT<S>* __restrict__ cu, const uint8_t* __restrict__ cls,
-            Geo g, Prm<R> P, int yshift)
+k_step_tile(const S* fA, S* fB, CuT<S>* cu, const uint8_t* __restrict__ cls, Geo g, Prm<R> P, int yshift)
 {
     __shared__ TileShared<R, TY> sh;
     tile_step<S, R, TY, MRT, UNI, false>(fA, fB, cu, cls, g, P, blockIdx.x * 32, (int)blockIdx.y * TY - yshift, sh);
@@ -522,6 +521,9 @@ template <typename S, typename R, int TY, bool MRT>
 __device__ __noinline__ void wall_tile(const S* fA, S* fB, CuT<S>* cu, const uint8_t* cls, const Geo& g, const Prm<R>& P,
                                        int bx, int by, TileShared<R, TY>& sh)
 {
+    fA = global_ptr(fA);
+    fB = global_ptr(fB);
+    cu = global_ptr(cu);
     const int y0 = by * TY - tile_shift(g.edge[3] == EDGE_LID, g.ny, TY);
     if (kLean<R> && P.uni != R(0))
         tile_step<S, R, TY, MRT, kLean<R>, true>(fA, fB, cu, cls, g, P, bx * 32, y0, sh);
@@ -546,10 +548,13 @@ union __align__(16) MarchShared {
 // of the interior (interior_tile).  One launch, which overlaps the end of the
 // step before it; as two launches on two streams between events, GB300, us per
 // step: 2048^2 FP32 209.0 -> 204.7, FP16 149.8 -> 147.0, 1024x2048
-// impact FP32 113.1 -> 111.9.
+// impact FP32 113.1 -> 111.9.  With plain loads (see after_previous_launch) and
+// the overlap, against loads through the read-only path without it: 2048^2 FP64
+// 1804 -> 1791, FP32 205 -> 202, 1024x2048 impact FP32 115 -> 113; 16-bit storage
+// see kPipeG16.
 template <typename S, typename R, int BLOCK, bool PREFETCH, int MINB, bool MRT, bool UNI>
 __global__ void __launch_bounds__(BLOCK, MINB)
-k_step_march(const S* __restrict__ fA, S* __restrict__ fB, CuT<S>* __restrict__ cu, const uint8_t* __restrict__ cls,
+k_step_march(const S* fA, S* fB, CuT<S>* cu, const uint8_t* __restrict__ cls,
              const uint32_t* __restrict__ walls, int nwalls, int strips, const __grid_constant__ Geo g,
              const __grid_constant__ Prm<R> P, int rows)
 {
