@@ -1457,7 +1457,7 @@ int tlb3_read_fields(tlb3_lattice* L, uint32_t mask, double* host_out)
     if ((rc = L->prec == TLB_FP32 ? read3_t<float>(L, stage) : read3_t<double>(L, stage))) return rc;
     int planes = 0;
     for (int q = 0; q < 11; q++) planes += (mask >> q) & 1u;
-    tlb::touch_host(host_out, (size_t)planes * N * sizeof(double));
+    tlb::ready_host(host_out, (size_t)planes * N * sizeof(double));
     size_t done = 0;
     for (int q = 0; q < 11; q++) {
         if (!(mask & (1u << q))) continue;

@@ -662,7 +662,7 @@ int tlb_read_fields(tlb_lattice* L, uint32_t mask, double* host_out)
     double* stage = (double*)(L->lay.inplace ? L->cpl() : L->bufB());
     size_t planes = 0;
     for (int q = 0; q < 10; q++) planes += (mask >> q) & 1u;
-    tlb::touch_host(host_out, planes * N * 8);
+    tlb::ready_host(host_out, planes * N * 8);
     size_t done = 0;
     for (int q = 0; q < 10;) {
         uint32_t sub = 0;

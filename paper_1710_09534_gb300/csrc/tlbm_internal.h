@@ -4,6 +4,7 @@
 #include <vector>
 #include "tlbm.h"
 #include "tlbm_device.cuh"
+#include "tlbm_host.h"
 #include "tlbm_ops.h"
 
 namespace tlb {
@@ -86,14 +87,13 @@ void batch_member_changed(tlb_batch* B);
 // batch steps still queued on it); TLB_OK for a lattice outside any batch.
 int batch_sync(tlb_batch* B);
 
-// Writes one byte of every page of a host buffer that is about to be filled by
-// copies from the device: the device takes the page faults of a fresh buffer
-// one by one (GB300, 170 MB of FP64 planes: 53 ms, after 5 ms of touching 1 ms).
-inline void touch_host(void* p, size_t bytes)
+// Readies the caller's buffer for copies from the device: maps its pages if it
+// is pageable memory (memory that CUDA knows has them).
+inline void ready_host(void* p, size_t bytes)
 {
-    volatile char* c = (volatile char*)p;
-    for (size_t i = 0; i < bytes; i += 4096) c[i] = 0;
-    if (bytes) c[bytes - 1] = 0;
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) == cudaSuccess && at.type == cudaMemoryTypeUnregistered)
+        (void)map_host_pages(p, bytes);
 }
 
 // Record an error message for tlb_last_error() and return `code`.
