@@ -338,15 +338,20 @@ constexpr bool kGReg3 = !kLo3<R>;
 // block's shared-memory stage (stride = block size, element = thread) that
 // the update fills by asynchronous copies at its start; ready() waits for
 // this thread's copies (STG 1) or for those of the whole block (STG 2; every
-// thread of the block calls it once, wherever it then is).
+// thread of the block calls it once, wherever it then is).  STG 3: global
+// memory through the read-only path (ordinary launches only).
 template <typename R, int STG>
 struct PopSrc {
     const R* b;  // plane 0 of the node
     long long pl;
-    __device__ __forceinline__ R operator()(int q) const { return b[q * pl]; }
+    __device__ __forceinline__ R operator()(int q) const
+    {
+        if constexpr (STG == 3) return __ldg(b + q * pl);
+        else return b[q * pl];
+    }
     __device__ __forceinline__ void ready() const
     {
-        if constexpr (STG != 0) asm volatile("cp.async.wait_all;" ::: "memory");
+        if constexpr (STG == 1 || STG == 2) asm volatile("cp.async.wait_all;" ::: "memory");
         if constexpr (STG == 2) asm volatile("barrier.sync 0;" ::: "memory");
     }
 };
@@ -603,8 +608,8 @@ __device__ __forceinline__ void cp_async(unsigned dst, const void* src)
     asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(dst), "l"(src), "n"(N) : "memory");
 }
 
-template <typename R, bool UNI, int STG>
-__device__ __forceinline__ void update3_node(const PopSrc<R, STG>& fs, const PopSrc<R, STG>& cs, R* __restrict__ fB,
+template <typename R, bool UNI, int STG, int STC>
+__device__ __forceinline__ void update3_node(const PopSrc<R, STG>& fs, const PopSrc<R, STC>& cs, R* __restrict__ fB,
                                              R* __restrict__ cu, const R* __restrict__ cpl,
                                              const R* __restrict__ mpl, uint32_t L, const Geo3& g, int x, int y,
                                              int z, long long o, const Prm3<R>& P)
@@ -714,12 +719,22 @@ __device__ __forceinline__ void update3_node(const PopSrc<R, STG>& fs, const Pop
     }
 }
 
+// The general FP64 update holds 2 blocks per SM and loads the populations of a
+// pair of directions after the stores of the pair before.  Plain loads wait for
+// those stores, loads through the read-only path do not, and here that is worth
+// more than the overlap with the launch before: GB300, us per step, dependent
+// launch with plain loads against this: 47x60x70 261, 230; 100x90x110 1140, 1032;
+// 161x96x160 2841, 2504; 128x64x128 1098, 1056.  The uniform one (3 blocks) is
+// faster dependent: 96x64x80 413, 417; 100x90x110 804, 810; FP32 reads its stage.
+template <typename R, bool UNI>
+constexpr bool kDependent3 = UNI || kStage3<R>;
+
 template <typename R, bool UNI>
 __global__ void __launch_bounds__(128, kLo3<R> ? (UNI ? TLB3_MINB32 : TLB3_MINB32_GEN) : (UNI ? TLB3_MINB : TLB3_MINB_GEN))
 k3_update(const R* fA, R* fB, R* cu, const R* cpl, const R* mpl, const uint32_t* __restrict__ lnk, Geo3 g,
           Prm3<R> P)
 {
-    tlb::after_previous_launch();
+    if constexpr (kDependent3<R, UNI>) tlb::after_previous_launch();
     NODE_OF_THREAD
     const long long PL = g.plane;
     if constexpr (kStage3<R>) {
@@ -750,8 +765,8 @@ k3_update(const R* fA, R* fB, R* cu, const R* cpl, const R* mpl, const uint32_t*
     } else {
         const uint32_t L = lnk[o];
         if (L & LNK_SOLID) return;
-        update3_node<R, UNI>(PopSrc<R, 0>{fA + o, PL}, PopSrc<R, 0>{cu + o, PL}, fB, cu, cpl, mpl, L, g, x,
-                             y, z, o, P);
+        update3_node<R, UNI>(PopSrc<R, kDependent3<R, UNI> ? 0 : 3>{fA + o, PL}, PopSrc<R, 0>{cu + o, PL}, fB, cu,
+                             cpl, mpl, L, g, x, y, z, o, P);
     }
 }
 
@@ -1138,10 +1153,16 @@ int update3_t(tlb3_lattice* L)
             return TLB_OK;
         }
     }
-    auto* k = L->uni ? &tlb3::k3_update<R, true> : &tlb3::k3_update<R, false>;
-    T3_CUDA(tlb::launch_dependent(k, grid3(L), 128, dyn, L->stream, (const R*)L->fcur<R>(), L->fspare<R>(), L->cu<R>(),
-                                  (const R*)L->cpl<R>(), (const R*)L->mpl<R>(), (const uint32_t*)L->lnk(), L->geo,
-                                  L->P<R>()));
+    if (L->uni || tlb3::kDependent3<R, false>) {
+        auto* k = L->uni ? &tlb3::k3_update<R, true> : &tlb3::k3_update<R, false>;
+        T3_CUDA(tlb::launch_dependent(k, grid3(L), 128, dyn, L->stream, (const R*)L->fcur<R>(), L->fspare<R>(),
+                                      L->cu<R>(), (const R*)L->cpl<R>(), (const R*)L->mpl<R>(),
+                                      (const uint32_t*)L->lnk(), L->geo, L->P<R>()));
+        return TLB_OK;
+    }
+    tlb3::k3_update<R, false><<<grid3(L), 128, dyn, L->stream>>>(L->fcur<R>(), L->fspare<R>(), L->cu<R>(), L->cpl<R>(),
+                                                                 L->mpl<R>(), L->lnk(), L->geo, L->P<R>());
+    T3_CUDA(cudaGetLastError());
     return TLB_OK;
 }
 
