@@ -193,8 +193,9 @@ int tlb_set_fields_device(tlb_lattice *lat, const double *c1, const double *c2,
                           const double *ux, const double *uy, const double *p);
 
 /* Advance n >= 0 time steps, asynchronously on the stream: one launch per
- * step, over tiles up to about 3.0, 1.4 and 0.75 million nodes in FP64, FP32
- * and 16-bit storage and in marching strips beyond; in-place lattices: the
+ * step, over tiles up to about 2.2, 0.35 and 0.3 million nodes in FP64, FP32
+ * and 16-bit storage (16-bit MRT: 2.2 million) and in marching strips beyond;
+ * in-place lattices: the
  * order-parameter pass, the interior kernel, the lid row if any, the
  * near-wall kernel, and after a last even step the in-place streaming.  The
  * near-wall launches of an in-place lattice run on a stream the lattice owns,
@@ -283,8 +284,8 @@ int64_t tlb_wall_nodes(tlb_lattice *lat);
  * A batch steps all its member lattices in lockstep, one launch per step: a
  * persistent kernel whose blocks take the members' near-wall tiles and (member,
  * strip, segment) tiles of the fused interior update from a shared counter, or,
- * when the members together have no more nodes than a lattice that tlb_step
- * steps by one kernel, one block per tile of that kernel (same per-node
+ * when the members together have no more than about 3.0, 1.2 and 0.75 million
+ * nodes (FP64, FP32, 16-bit storage), one block per tile (same per-node
  * arithmetic as tlb_step, so a member's result does not depend on the rest of
  * the batch).  Pairs of steps run as one captured CUDA graph on the batch's
  * stream.

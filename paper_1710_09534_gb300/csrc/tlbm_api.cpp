@@ -602,7 +602,7 @@ int tlb_step(tlb_lattice* L, int64_t n)
     if (!L->have_params || !L->have_fields) return fail(TLB_ESTATE, "set_params and set_fields before step");
     if (L->batch) return fail(TLB_ESTATE, "lattice belongs to a batch: step the batch");
     if (L->lay.inplace) return step_inplace(L, n);
-    const bool tile = L->ops->use_tile(L->n());
+    const bool tile = L->ops->use_tile(L->n(), false);
     for (int64_t s = 0; s < n; s++) {
         rc = step_launches(
             L, false, [] { return cudaSuccess; },

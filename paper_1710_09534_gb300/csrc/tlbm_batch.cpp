@@ -109,7 +109,7 @@ int rebuild(tlb_batch* B)
     int64_t wall_nodes = 0;
     int64_t nodes = 0;
     for (const tlb_lattice* L : B->members) nodes += L->n();
-    B->tile = B->ops->use_tile(nodes);
+    B->tile = B->ops->use_tile(nodes, true);
     // columns and rows of an item
     const int tx = B->tile ? 64 : (B->variant == 0 ? 64 : 128) - 4;
     for (size_t i = 0; i < B->members.size(); i++) {
@@ -424,7 +424,7 @@ int tlb_batch_tune(tlb_batch* B, int trial_steps_n, void* dev_scratch, int64_t s
     int64_t nodes = 0;
     for (const tlb_lattice* L : B->members) nodes += L->n();
     // (one-tile blocks have one shape: the current one is timed and kept)
-    const bool one = B->ops->use_tile(nodes);
+    const bool one = B->ops->use_tile(nodes, true);
     const int current[3] = {B->variant == 0 ? 64 : 128, B->rows_small, B->rows_large};
     const int (*cand)[3] = one ? &current : shapes;
     for (int i = 0; rc == TLB_OK && i < (one ? 1 : (int)(sizeof shapes / sizeof shapes[0])); i++) {

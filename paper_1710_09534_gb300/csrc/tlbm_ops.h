@@ -19,7 +19,7 @@ struct Ops {
     // the same step by tiles (k_step_tile), for lattices (or batches) of few enough nodes (use_tile)
     cudaError_t (*tile)(const void* fA, void* fB, void* cu, const uint8_t* cls, const Geo& g, const Prm<double>& P,
                         cudaStream_t s);
-    bool (*use_tile)(long long nodes);
+    bool (*use_tile)(long long nodes, bool batch);
     cudaError_t (*init)(void* fA, void* cu, const uint8_t* cls, const double* c1, const double* c2,
                         const double* ux, const double* uy, const double* p, const Geo& g,
                         const Prm<double>& P, cudaStream_t s);

@@ -123,6 +123,12 @@ inline int sm_count()
 // often as it gained (2048x1024 123.6, 126.0; 2048^2 237.6, 231.5) and is off.
 // In-place FP64 takes the one-wave rule, in which its halo is cheap (c comes
 // from planes): 2048x1024 1016 -> 889.
+// A lattice of less than one wave of 16-row segments takes shorter ones: of 4 to
+// 15 rows (two buffers), the length with the fewest row iterations in all, waves
+// times rows and halo; halving until the blocks exceed the resident ones could end
+// just beyond a wave.  GB300, us per step, halving against this: FP32 777^2 44.9,
+// 36.7; 500x1000 38.6, 30.4; 860^2 48.8, 42.5; FP16 860^2 33.2, 30.3; 1255x695 42.1, 36.5.
+constexpr int kMarchHalo = 4;  // halo rows of a segment of k_step_march
 inline int rows_for(const Geo& g, int tx, int rows, int per_sm, bool one_wave, int halo)
 {
     if (!TLB_ADAPTIVE_ROWS) return rows;
@@ -144,6 +150,13 @@ inline int rows_for(const Geo& g, int tx, int rows, int per_sm, bool one_wave, i
         int best = rows;
         for (int r = 12; r <= 24; r++)
             if (cost(r) < 0.98 * cost(rows) && cost(r) < cost(best)) best = r;
+        return best;
+    }
+    if (halo == kMarchHalo) {
+        auto iterations = [&](int r) { return (blocks(r) + slots - 1) / slots * (r + halo); };
+        int best = rows;
+        for (int r = rows - 1; r >= 4; r--)
+            if (iterations(r) < iterations(best)) best = r;
         return best;
     }
     while (rows > 4 && blocks(rows) < slots) rows /= 2;
@@ -168,7 +181,7 @@ struct OpsImpl {
         static_assert(BLOCK == 32 * kWallTY, "a block takes a strip segment or a near-wall tile");
         // equal densities and viscosities: the uniform-property update
         const bool uni = Pd.uni != 0.0;
-        const int rows = rows_for(g, TX, ROWS, uni ? kMinBUni : MINB, std::is_same<R, double>::value, 4);
+        const int rows = rows_for(g, TX, ROWS, uni ? kMinBUni : MINB, std::is_same<R, double>::value, kMarchHalo);
         const int strips = (g.nx + TX - 1) / TX, segs = (g.ny + rows - 1) / rows;
         auto* k = uni ? &k_step_march<S, R, BLOCK, PREFETCH, kMinBUni, MRT, true>
                       : &k_step_march<S, R, BLOCK, PREFETCH, MINB, MRT, false>;
@@ -206,18 +219,27 @@ struct OpsImpl {
             return launch_tile<8, 3>(fA, fB, cu, cls, g, Pd, s);
         }
     }
-    // One launch per step up to these sizes; beyond them the state no longer
-    // stays in L2 (FP32, 16-bit: the marching kernel's loads one row ahead cover
-    // more of the memory latency) or the near-wall launch is hidden (FP64).
-    // GB300, us per step, marching and near-wall kernels against this one: FP64
-    // 128x64 45.2, 16.5; 512x256 142, 102; 1024x1024 565, 494; 1024x2048 1339,
-    // 1190; 2048x2048 1940, 1938.  FP32 128x64 13.5, 3.7; 512x256 20.6, 9.7;
-    // 1024x1024 68.2, 64.8; 1200x1100 91.4, 88.0; 1024x2048 114, 127.  FP16
-    // 128x64 12.6, 3.9; 512x256 22.1, 10.2; 512x1024 31.7, 26.4; 1024x1024 48.2,
-    // 53.8.
-    static bool use_tile(long long nodes)
+    // One launch per step by tiles up to these sizes; beyond them the marching
+    // kernel's loads one row ahead cover more of the memory latency (FP32, 16-bit)
+    // or its halo is the smaller one (FP64).  GB300, us per step, k_step_tile
+    // against k_step_march, uniform and general update: FP64 1000^2 454, 473 and
+    // 574, 618; 1400^2 853, 847 and 1081, 1110; 1600^2 1095, 1043 and 1385, 1369.
+    // FP32 500^2 14.0, 15.9 and 15.9, 16.5; 600^2 20.9, 21.4 and 23.5, 21.5; 777^2
+    // 40.1, 36.7 and 43.1, 36.7; 1180^2 81.6, 73.5 and 86.6, 75.1.  FP16 500^2 13.7,
+    // 14.3 and 14.9, 15.9; 600^2 18.7, 17.0 and 20.2, 18.7; 860^2 40.2, 30.3 and 42.9,
+    // 32.6.  MRT: FP64 1400^2 1247, 1281; 1600^2 1601, 1578; FP32 500^2 21.4, 25.3;
+    // 600^2 31.7, 30.4; 16-bit storage, whose dense update leaves the marching kernel
+    // no loads ahead, later: FP16 860^2 58.3, 57.5; 1300^2 123.8, 124.1; 1500^2 162,
+    // 168; 1730^2 215, 208; BF16 1180^2 98, 99; 1500^2 154, 158; 1730^2 205, 196.
+    // Batches (their members' nodes together; the persistent kernel against
+    // k_batch_tile): FP64 1.9 million 1242, 862; FP32 0.98 83.6, 74.9; 1.43 95.4, 103;
+    // FP16 0.72 68, 52; 1.43 76, 93.
+    static bool use_tile(long long nodes, bool batch)
     {
-        return nodes <= (std::is_same<S, double>::value ? 3000000 : std::is_same<S, float>::value ? 1400000 : 750000);
+        if (std::is_same<S, double>::value) return nodes <= (batch ? 3000000 : 2200000);
+        if (std::is_same<S, float>::value) return nodes <= (batch ? 1200000 : 350000);
+        if (batch) return nodes <= 750000;
+        return nodes <= (kDenseMrt<S, MRT> ? 2200000 : 300000);
     }
     static cudaError_t init(void* fA, void* cu, const uint8_t* cls, const double* c1, const double* c2,
                             const double* ux, const double* uy, const double* p, const Geo& g,
