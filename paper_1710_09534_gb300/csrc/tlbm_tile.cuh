@@ -505,10 +505,12 @@ k_read_fields(const S* __restrict__ fA, const uint8_t* __restrict__ cls, double*
 
 template <typename S, typename R, int TY, int MINB, bool MRT, bool UNI>
 __global__ void __launch_bounds__(32 * TY, MINB)
-k_step_tile(const S* fA, S* fB, CuT<S>* cu, const uint8_t* __restrict__ cls, Geo g, Prm<R> P, int yshift)
+k_step_tile(const S* fA, S* fB, CuT<S>* cu, const uint8_t* __restrict__ cls, Geo g, Prm<R> P, int yshift, int first)
 {
     __shared__ TileShared<R, TY> sh;
-    tile_step<S, R, TY, MRT, UNI, false>(fA, fB, cu, cls, g, P, blockIdx.x * 32, (int)blockIdx.y * TY - yshift, sh);
+    int by = (int)blockIdx.y + first;  // rows of tiles from row `first` on, cyclically
+    by -= by >= (int)gridDim.y ? (int)gridDim.y : 0;
+    tile_step<S, R, TY, MRT, UNI, false>(fA, fB, cu, cls, g, P, blockIdx.x * 32, by * TY - yshift, sh);
 }
 
 // ---------------------------------------------------------------------------
