@@ -106,10 +106,19 @@ int rebuild(tlb_batch* B)
                      [&](int a, int b) { return B->members[a]->n() > B->members[b]->n(); });
     std::vector<tlb::TileItem> tiles;
     std::vector<tlb::WallItem> walls;
-    int64_t wall_nodes = 0;
-    int64_t nodes = 0;
-    for (const tlb_lattice* L : B->members) nodes += L->n();
-    B->tile = B->ops->use_tile(nodes, true);
+    int64_t wall_nodes = 0, nodes = 0, shape_tiles = 0, block_tiles = 0;
+    for (const tlb_lattice* L : B->members) {
+        nodes += L->n();
+        wall_nodes += L->nlist;
+        shape_tiles += tiles_of(B->variant, rows_for(B, L), L->nx, L->ny);
+        block_tiles += (int64_t)((L->nx + 63) / 64) * ((L->ny + tlb::kBatchTY - 1) / tlb::kBatchTY);
+    }
+    // the capacity asked for is that of the configured shape, however the batch
+    // is stepped (a near-wall tile holds at least one near-wall node)
+    if (shape_tiles > B->max_tiles || wall_nodes > B->max_wall)
+        return err(TLB_ENOMEM, "batch needs %lld tiles and %lld wall nodes; capacity %lld and %lld",
+                   (long long)shape_tiles, (long long)wall_nodes, (long long)B->max_tiles, (long long)B->max_wall);
+    B->tile = B->ops->use_tile(nodes, true) && block_tiles <= B->max_tiles;
     // columns and rows of an item
     const int tx = B->tile ? 64 : (B->variant == 0 ? 64 : 128) - 4;
     for (size_t i = 0; i < B->members.size(); i++) {
@@ -127,12 +136,7 @@ int rebuild(tlb_batch* B)
             for (int bx = 0; bx < nbx; bx++) tiles.push_back({i, bx, by});
         if (!B->tile)
             for (uint32_t p : tlb::wall_tiles(L->hlist, L->geo, B->variant == 0 ? 2 : 4)) walls.push_back({i, p});
-        wall_nodes += L->nlist;
     }
-    // (a near-wall tile holds at least one near-wall node)
-    if ((int64_t)tiles.size() > B->max_tiles || wall_nodes > B->max_wall)
-        return err(TLB_ENOMEM, "batch needs %zu tiles and %lld wall nodes; capacity %lld and %lld", tiles.size(),
-                   (long long)wall_nodes, (long long)B->max_tiles, (long long)B->max_wall);
     tlb::BatchCounters c{(int)tiles.size(), (int)walls.size(), 0, 0};
     if (!descs.empty())
         B_CUDA(cudaMemcpyAsync(B->ws + B->lay.desc, descs.data(), descs.size(), cudaMemcpyHostToDevice, B->stream));
