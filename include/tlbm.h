@@ -302,13 +302,14 @@ int64_t tlb_wall_nodes(tlb_lattice *lat);
  * tlb_batch_remove synchronizes the batch stream.  tlb_batch_step advances
  * every member n steps, asynchronously.  tlb_batch_config sets the tile shape
  * (threads 64 or 128; row segments rows_small for members with ny <=
- * small_ny, rows_large otherwise); batches stepped by one block per tile have
- * one shape only and keep the setting for when they grow.
+ * small_ny, rows_large otherwise); batches stepped by one block per tile
+ * have no use for it until they grow.
  *
  * tlb_batch_tune times 8 candidate shapes on the batch's own members,
  * trial_steps + 2 trial steps each, keeps the fastest and reports {threads,
- * rows_small, rows_large, small_ny} and its time per step (one block per tile:
- * times and reports the current setting).  It leaves every
+ * rows_small, rows_large, small_ny} and the batch's time per step with it (a
+ * batch stepped by one block per tile: the time of those steps; the shape is
+ * for when it grows).  It leaves every
  * member's state as it was: each trial step reads the members' current
  * distributions and writes their spare buffer without making it current, and
  * the c_i u planes of Eq. 19 (the only state a step updates in place) are

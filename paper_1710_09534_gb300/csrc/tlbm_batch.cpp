@@ -71,6 +71,7 @@ struct tlb_batch {
     bool dirty = true;
     int64_t n_tiles = 0, n_wall = 0;
     bool tile = false;            // the members together are small enough for one-tile blocks (k_batch_tile)
+    bool shape_trials = false;    // the tuner is timing shapes: no one-tile blocks
     int grid = 0;
     cudaGraphExec_t graph = nullptr;
     int graph_variant = -1, graph_grid = 0;
@@ -118,7 +119,7 @@ int rebuild(tlb_batch* B)
     if (shape_tiles > B->max_tiles || wall_nodes > B->max_wall)
         return err(TLB_ENOMEM, "batch needs %lld tiles and %lld wall nodes; capacity %lld and %lld",
                    (long long)shape_tiles, (long long)wall_nodes, (long long)B->max_tiles, (long long)B->max_wall);
-    B->tile = B->ops->use_tile(nodes, true) && block_tiles <= B->max_tiles;
+    B->tile = !B->shape_trials && B->ops->use_tile(nodes, true) && block_tiles <= B->max_tiles;
     // columns and rows of an item
     const int tx = B->tile ? 64 : (B->variant == 0 ? 64 : 128) - 4;
     for (size_t i = 0; i < B->members.size(); i++) {
@@ -425,18 +426,21 @@ int tlb_batch_tune(tlb_batch* B, int trial_steps_n, void* dev_scratch, int64_t s
     double best = 1e30;
     int best_i = 0;
     rc = copy_cu(B, (char*)dev_scratch, true);
-    int64_t nodes = 0;
-    for (const tlb_lattice* L : B->members) nodes += L->n();
-    // (one-tile blocks have one shape: the current one is timed and kept)
-    const bool one = B->ops->use_tile(nodes, true);
-    const int current[3] = {B->variant == 0 ? 64 : 128, B->rows_small, B->rows_large};
-    const int (*cand)[3] = one ? &current : shapes;
-    for (int i = 0; rc == TLB_OK && i < (one ? 1 : (int)(sizeof shapes / sizeof shapes[0])); i++) {
-        B->variant = cand[i][0] == 64 ? 0 : 1;
-        B->rows_small = cand[i][1];
-        B->rows_large = cand[i][2];
-        B->small_ny = one ? saved[3] : 128;
+    // the shapes, and after them (index n_shapes) the best one as the batch is
+    // stepped with it, which by one-tile blocks is another kernel
+    const int n_shapes = (int)(sizeof shapes / sizeof shapes[0]);
+    for (int i = 0; rc == TLB_OK && i <= n_shapes; i++) {
+        const int* shape = shapes[i < n_shapes ? i : best_i];
+        B->variant = shape[0] == 64 ? 0 : 1;
+        B->rows_small = shape[1];
+        B->rows_large = shape[2];
+        B->small_ny = 128;
+        B->shape_trials = i < n_shapes;
         B->dirty = true;
+        if (i == n_shapes) {
+            if ((rc = rebuild(B)) || !B->tile) break;
+            best = 1e30;
+        }
         if ((rc = trial_steps(B, 2))) break;  // warm-up (also rebuilds the lists)
         cudaError_t ce = cudaEventRecord(e0, B->stream);
         if (ce == cudaSuccess && (rc = trial_steps(B, trial_steps_n)) == TLB_OK) ce = cudaEventRecord(e1, B->stream);
@@ -450,9 +454,10 @@ int tlb_batch_tune(tlb_batch* B, int trial_steps_n, void* dev_scratch, int64_t s
         }
         if (ms / trial_steps_n < best) {
             best = ms / trial_steps_n;
-            best_i = i;
+            if (i < n_shapes) best_i = i;
         }
     }
+    B->shape_trials = false;
     // put back the c_i u planes the trial steps overwrote (the distributions
     // of the current buffer were only read)
     const int rc_restore = copy_cu(B, (char*)dev_scratch, false);
@@ -468,13 +473,13 @@ int tlb_batch_tune(tlb_batch* B, int trial_steps_n, void* dev_scratch, int64_t s
         return rc ? rc : rc_restore;
     }
     if (es != cudaSuccess) return err(TLB_ECUDA, "batch stream: %s", cudaGetErrorString(es));
-    B->variant = cand[best_i][0] == 64 ? 0 : 1;
-    B->rows_small = cand[best_i][1];
-    B->rows_large = cand[best_i][2];
+    B->variant = shapes[best_i][0] == 64 ? 0 : 1;
+    B->rows_small = shapes[best_i][1];
+    B->rows_large = shapes[best_i][2];
     if (out_config) {
-        out_config[0] = cand[best_i][0];
-        out_config[1] = cand[best_i][1];
-        out_config[2] = cand[best_i][2];
+        out_config[0] = shapes[best_i][0];
+        out_config[1] = shapes[best_i][1];
+        out_config[2] = shapes[best_i][2];
         out_config[3] = B->small_ny;
     }
     if (out_ms_per_step) *out_ms_per_step = best;
