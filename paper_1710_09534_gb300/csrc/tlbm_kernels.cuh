@@ -330,7 +330,7 @@ __device__ __forceinline__ void collide_all(Collider<R, UNI, MRT>& col, const R 
     };
     if constexpr (MRT) {
         col.moments_of_g(gv);
-        R p1[4], p2[4];  // f_k - f_k-bar of the four opposite pairs
+        R p1[4], p2[4], q1[4], q2[4];  // f_k -+ f_k-bar of the four opposite pairs
         static_for<0, 4>([&](auto pc) {
             constexpr int I = decltype(pc)::value, K = pair_dir(I), KB = opp(K);
             R a1, a2, b1, b2;
@@ -338,9 +338,11 @@ __device__ __forceinline__ void collide_all(Collider<R, UNI, MRT>& col, const R 
             load(std::integral_constant<int, KB>{}, b1, b2);
             p1[I] = a1 - b1;
             p2[I] = a2 - b2;
+            q1[I] = a1 + b1;
+            q2[I] = a2 + b2;
         });
-        col.flux_of_f(p1[0] + (p1[2] + p1[3]), p1[1] + (p1[2] - p1[3]), p2[0] + (p2[2] + p2[3]),
-                      p2[1] + (p2[2] - p2[3]));
+        col.moments_of_f(p1[0] + (p1[2] + p1[3]), p1[1] + (p1[2] - p1[3]), p2[0] + (p2[2] + p2[3]),
+                         p2[1] + (p2[2] - p2[3]), (q1[0] + q1[1]) + (q1[2] + q1[3]), (q2[0] + q2[1]) + (q2[2] + q2[3]));
     }
     R d1 = R(0), d2 = R(0);  // sum_k (f_k - o'_k) over the moving directions
     // the directions go in opposite pairs (k, k-bar), which share most of
