@@ -83,7 +83,7 @@ struct Prm3 {
     // uniform properties (rho, nu equal in the three fluids)
     R rho0, irho, hirho, prho;  // rho, 1/rho, 1/(2 rho), -rho/4
     R itg0, omtg0, kG0, Kw0[2], Rw0[2], p3tg0, Gc[2];
-    R kqs[2], kl2[2], kl3[2];  // kq + sq, 2 kl, -3 kl (FP64)
+    R kqs[2], kl1[2], kl2[2], kl3[2];  // kq + sq, kl (tripled_exactly), 2 kl1, -3 kl1 (FP64)
 };
 
 // FP64 forms with fewer instructions, as in two dimensions (tlb::kLean): Q_i
@@ -158,8 +158,8 @@ __device__ __forceinline__ void chem_pot(const Prm3<R>& P, R c1, R c2, R l6c1, R
     const R c3 = R(1.0) - c1 - c2;
     const R t = P.kT * (c1 * c2) * c3;
     if constexpr (kLean3<R>) {
-        mu1 = fma(-P.kd6[0], l6c1, fma(c1, fma(c1, fma(c1, P.kl2[0], P.kl3[0]), P.kl[0]), -t));
-        mu2 = fma(-P.kd6[1], l6c2, fma(c2, fma(c2, fma(c2, P.kl2[1], P.kl3[1]), P.kl[1]), -t));
+        mu1 = fma(-P.kd6[0], l6c1, fma(c1, fma(c1, fma(c1, P.kl2[0], P.kl3[0]), P.kl1[0]), -t));
+        mu2 = fma(-P.kd6[1], l6c2, fma(c2, fma(c2, fma(c2, P.kl2[1], P.kl3[1]), P.kl1[1]), -t));
         return;
     }
     const R h1 = c1 * fma(c1, fma(R(2.0), c1, -R(3.0)), R(1.0));
@@ -1355,8 +1355,9 @@ int tlb3_set_params(tlb3_lattice* L, const tlb_params* p)
         P.kq[i] = 3.0 * w36 / tau[i];
         P.sq[i] = 3.0 * w36 * (1.0 - 0.5 / tau[i]);
         P.kqs[i] = P.kq[i] + P.sq[i];
-        P.kl2[i] = 2.0 * P.kl[i];
-        P.kl3[i] = -3.0 * P.kl[i];
+        P.kl1[i] = tlb::tripled_exactly(P.kl[i]);
+        P.kl2[i] = 2.0 * P.kl1[i];
+        P.kl3[i] = -3.0 * P.kl1[i];
     }
     // uniform properties: the constants of the UNI update
     P.rho0 = rho[0];

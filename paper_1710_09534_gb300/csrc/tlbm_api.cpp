@@ -440,8 +440,9 @@ int tlb_set_params(tlb_lattice* L, const tlb_params* p)
         P.aM6[i] = P.aM[i] / 6.0;
         P.K3w3[i] = 3.0 * P.Kw3[i];
         P.kqs[i] = P.kq[i] + P.ks[i];
-        P.Kl2[i] = 2.0 * P.Kl[i];
-        P.Kl3[i] = -3.0 * P.Kl[i];
+        P.Kl1[i] = tlb::tripled_exactly(P.Kl[i]);
+        P.Kl2[i] = 2.0 * P.Kl1[i];
+        P.Kl3[i] = -3.0 * P.Kl1[i];
     }
     P.rho23 = -2.0 / 3.0 * p->rho3;
     P.kp3 = 0.6 * P.p3tg3;

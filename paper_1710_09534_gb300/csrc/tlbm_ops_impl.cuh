@@ -70,6 +70,7 @@ inline Prm<R> cast_prm(const Prm<double>& d)
         r.ks[i] = R(d.ks[i]);
         r.K3w3[i] = R(d.K3w3[i]);
         r.kqs[i] = R(d.kqs[i]);
+        r.Kl1[i] = R(d.Kl1[i]);
         r.Kl2[i] = R(d.Kl2[i]);
         r.Kl3[i] = R(d.Kl3[i]);
         r.qa[i][0] = R(d.qa[i][0]);
