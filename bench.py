@@ -135,8 +135,8 @@ def parse():
     return ap.parse_args()
 
 
-# the sources that define the two-buffer interior kernel and its launch
-INTERIOR_SOURCES = ("tlbm_device.cuh", "tlbm_kernels.cuh", "tlbm_ops.h", "tlbm_ops_impl.cuh",
+# the sources that define the two-buffer interior kernel (k_step_march) and its launch
+INTERIOR_SOURCES = ("tlbm_device.cuh", "tlbm_kernels.cuh", "tlbm_tile.cuh", "tlbm_ops.h", "tlbm_ops_impl.cuh",
                     "tlbm_f64.cu", "tlbm_f32.cu", "tlbm_f16.cu", "tlbm_bf16.cu")
 
 
