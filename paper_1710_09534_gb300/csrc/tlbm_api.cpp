@@ -171,14 +171,17 @@ int prof_fold(tlb_lattice* L)
     if (L->ev_used == 0) return TLB_OK;
     TLB_CUDA(cudaEventSynchronize(L->ev[4 * (L->ev_used - 1) + 1]));
     TLB_CUDA(cudaEventSynchronize(L->ev[4 * (L->ev_used - 1) + 3]));
+    const bool wall = L->lay.inplace && L->nlist > 0;
     for (int i = 0; i < L->ev_used; i++) {
         float a = 0, b = 0;
         TLB_CUDA(cudaEventElapsedTime(&a, L->ev[4 * i], L->ev[4 * i + 1]));
         TLB_CUDA(cudaEventElapsedTime(&b, L->ev[4 * i + 2], L->ev[4 * i + 3]));
         L->prof_ms[0] += a;
-        L->prof_ms[1] += b;
         L->prof_n[0] += 1;
-        L->prof_n[1] += L->lay.inplace && L->nlist > 0 ? 1 : 0;
+        if (wall) {  // without a near-wall launch its two events follow each other
+            L->prof_ms[1] += b;
+            L->prof_n[1] += 1;
+        }
     }
     L->ev_used = 0;
     return TLB_OK;
