@@ -90,7 +90,7 @@ struct Prm3 {
 // from the old c_i u directly, the diagonal links' R_X and P_X as half the axis
 // links', the rest direction as 6 axis links with e = 0 less its 3 p, Eq. 8's
 // lambda_i in the Horner form (update 352 -> 340, mu 51 -> 49 instructions per
-// node; GB300, 96x64x80: 436 -> 420 us per step).
+// node; GB300, 96x64x80: 436 -> 420 us per step, 414 with overlapping launches).
 template <typename R>
 constexpr bool kLean3 = sizeof(R) == 8;
 

@@ -133,8 +133,8 @@ __device__ __forceinline__ bool fluidlike(int s) { return s == ST_FLUID || s == 
 //           vanishes exactly (with the rounding of 3 Kl it did not, and in three
 //           dimensions the pressure's rms error was 1.21 times as large)
 // FP32 arithmetic keeps its forms (16-bit storage rounds to them each step).
-// GB300, FP64: 2048^2 1905 -> 1780 us per step; 128x64 (near-wall nodes with
-// the uniform update too) 16.5 -> 13.3.
+// GB300, FP64: 2048^2 1905 -> 1767 us per step; 128x64 (near-wall nodes with
+// the uniform update too) 16.5 -> 13.4.
 template <typename R>
 constexpr bool kLean = sizeof(R) == 8;
 

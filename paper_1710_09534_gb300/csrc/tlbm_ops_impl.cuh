@@ -209,9 +209,9 @@ struct OpsImpl {
     // Tile height and resident blocks, GB300, us per step (4 x 2: TY = 4 at 2
     // blocks per SM, and so on):
     //   FP64 (bound by the FP64 unit, so by the busiest SM): short tiles while
-    //     they spread over more SMs: 128x64 16.5 (4 x 2), 23.8 (8 x 2); 250x150
-    //     26.5, 27.5; 240x280 55.9, 56.1; from about 4 short tiles per SM on, the
-    //     smaller frame: 512x512 150, 132; 1024x1024 550, 494.
+    //     they spread over more SMs: 200^2 35.2 (4 x 2), 42.0 (8 x 2); 160^2 20.7,
+    //     19.8; 240x280 43.6, 42.5; from about 4 short tiles per SM on, the smaller
+    //     frame: 400x300 73.0, 72.0; 512^2 141, 121; 1000^2 506, 454.
     //   FP32 and 16-bit storage: TY = 8; a third block per SM (80 registers)
     //     pays once the grid exceeds 4 tiles per SM: FP32 240x280 5.8 (8 x 2),
     //     7.4 (8 x 3); 512x256 9.7, 10.2; 512x512 16.2, 14.0; 1024x1024 69.5, 64.8.

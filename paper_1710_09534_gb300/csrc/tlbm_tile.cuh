@@ -19,7 +19,7 @@
 // (programmatic dependent launch: a block classifies its sites while the
 // previous step finishes, then waits for it; 128x64 FP32 6.2 -> 3.7 us per
 // step).  GB300, us per step, the two kernels against this one: 128x64 FP64
-// 45.2 -> 16.5, FP32 13.5 -> 3.7; 512x256 with a lid FP32 20.6 -> 9.7.
+// 45.2 -> 13.4, FP32 13.5 -> 3.7; 512x256 with a lid FP32 20.6 -> 9.3.
 //
 // The arithmetic of every node is that of the other two kernels, operation by
 // operation: interior nodes use the column sums (ColRings), the others the
@@ -549,8 +549,8 @@ union __align__(16) MarchShared {
 // near-wall nodes of a straight wall are two rows), the others a strip segment
 // of the interior (interior_tile).  One launch, which overlaps the end of the
 // step before it; as two launches on two streams between events, GB300, us per
-// step: 2048^2 FP32 209.0 -> 204.7, FP16 149.8 -> 147.0, 1024x2048
-// impact FP32 113.1 -> 111.9.  With plain loads (see after_previous_launch) and
+// step: 2048^2 FP32 209.0 -> 200.1, FP16 149.8 -> 142.4, 1024x2048
+// impact FP32 113.1 -> 110.5.  With plain loads (see after_previous_launch) and
 // the overlap, against loads through the read-only path without it: 2048^2 FP64
 // 1804 -> 1791, FP32 205 -> 202, 1024x2048 impact FP32 115 -> 113; 16-bit storage
 // see kPipeG16.
