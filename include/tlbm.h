@@ -195,9 +195,9 @@ int tlb_set_fields_device(tlb_lattice *lat, const double *c1, const double *c2,
 /* Advance n >= 0 time steps, asynchronously on the stream: one launch per
  * step, over tiles up to about 2.2, 0.35 and 0.3 million nodes in FP64, FP32
  * and 16-bit storage (16-bit MRT: 2.2 million) and in marching strips beyond;
- * in-place lattices: the
- * order-parameter pass, the interior kernel, the lid row if any, the
- * near-wall kernel, and after a last even step the in-place streaming.  The
+ * in-place lattices: the order-parameter pass, the interior kernel, the lid row
+ * if any, the near-wall kernel, and after a last even step the in-place
+ * streaming.  The
  * near-wall launches of an in-place lattice run on a stream the lattice owns,
  * ordered after the step's earlier work and joined back into the caller's
  * stream before the step ends, so work the caller queues after tlb_step sees
@@ -213,8 +213,9 @@ int tlb_sync(tlb_lattice *lat, int64_t timeout_ms);
 /* Macroscopic fields of the current state as FP64 planes of nx*ny, in the
  * order of the set bits of field_mask (TLB_F_*): c1, c2, c3, rho, ux, uy, p,
  * mu1, mu2, mu3.  Solid nodes read 0; the lid row reads the row below it with
- * u = (U0, 0).  host_out receives popcount(field_mask)*nx*ny doubles.
- * Synchronizes the stream. */
+ * u = (U0, 0).  host_out receives popcount(field_mask)*nx*ny doubles, written
+ * in stream order: until the stream reaches this call, work queued before it
+ * may still read from the buffer.  Synchronizes the stream. */
 int tlb_read_fields(tlb_lattice *lat, uint32_t field_mask, double *host_out);
 
 /* The same into device memory (dev_out: popcount(field_mask)*nx*ny doubles);

@@ -92,7 +92,9 @@ int batch_sync(tlb_batch* B);
 inline void ready_host(void* p, size_t bytes)
 {
     cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, p) == cudaSuccess && at.type == cudaMemoryTypeUnregistered)
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess)
+        (void)cudaGetLastError();  // not the error of the launches that follow
+    else if (at.type == cudaMemoryTypeUnregistered)
         (void)map_host_pages(p, bytes);
 }
 
